@@ -170,10 +170,6 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
     return c;
 }
 
-__device__ __forceinline__ float word_to_tau(uint32_t w) {
-    return __fmul_rn((float)(w >> 8), 0x1p-24f);   // exact: 24-bit integer times 2^-24
-}
-
 // Mesh-colour cell: the micro-triangle of the N-subdivided triangle that
 // holds barycentrics (b1, b2).  Grid vertex (i, j), i + j <= N, sits at
 // barycentrics (1 - (i+j)/N, i/N, j/N) and has index j(N+1) - j(j-1)/2 + i.
@@ -184,32 +180,27 @@ struct Cell {
 };
 
 __device__ __forceinline__ int texel_index(int N, int i, int j) {
-    return j * (N + 1) - ((j * (j - 1)) >> 1) + i;
+    return ((j * (2 * N + 3 - j)) >> 1) + i;   // j (N + 1) - j (j - 1) / 2 + i
 }
 
+// Rounding towards minus infinity into int32 saturates (NaN gives 0), so the
+// clamps also hold for barycentrics outside the triangle; the corner
+// indices follow from the cell's first one: row j + 1 starts N + 1 - j
+// texels after the same column of row j.
 __device__ __forceinline__ Cell find_cell(int N, float b1, float b2) {
     const float Nf = (float)N;
     const float u = __fmul_rn(Nf, b1), v = __fmul_rn(Nf, b2);
-    const float fi = floorf(u), fj = floorf(v);
-    const int i = fi < 0.0f ? 0 : (fi > (float)(N - 1) ? N - 1 : (int)fi);
-    const int jmax = N - 1 - i;
-    const int j = fj < 0.0f ? 0 : (fj > (float)jmax ? jmax : (int)fj);
+    const int i = max(0, min(__float2int_rd(u), N - 1));
+    const int j = max(0, min(__float2int_rd(v), N - 1 - i));
     const float fu = __fsub_rn(u, (float)i), fv = __fsub_rn(v, (float)j);
     Cell c;
     c.lower = (__fadd_rn(fu, fv) <= 1.0f) || (i + j == N - 1);
-    if (c.lower) {
-        c.k0 = texel_index(N, i, j);
-        c.k1 = texel_index(N, i + 1, j);
-        c.k2 = texel_index(N, i, j + 1);
-        c.wa = fu;
-        c.wb = fv;
-    } else {
-        c.k0 = texel_index(N, i + 1, j + 1);
-        c.k1 = texel_index(N, i, j + 1);
-        c.k2 = texel_index(N, i + 1, j);
-        c.wa = __fsub_rn(1.0f, fu);
-        c.wb = __fsub_rn(1.0f, fv);
-    }
+    const int k = texel_index(N, i, j), row = N + 1 - j;
+    c.k0 = c.lower ? k : k + row + 1;
+    c.k1 = k + (c.lower ? 1 : row);
+    c.k2 = k + (c.lower ? row : 1);
+    c.wa = c.lower ? fu : __fsub_rn(1.0f, fu);
+    c.wb = c.lower ? fv : __fsub_rn(1.0f, fv);
     return c;
 }
 
@@ -223,13 +214,16 @@ struct Frag {
     float q1, q2, rho;
 };
 
-__device__ __forceinline__ Frag make_frag(long long e0, long long e1, long long e2, float k0, float k1, float k2) {
+__device__ __forceinline__ Frag edge_frag(float e0, float e1, float e2, float k0, float k1, float k2) {
     Frag f;
-    const float q0 = __fmul_rn(__ll2float_rn(e0), k0);
-    f.q1 = __fmul_rn(__ll2float_rn(e1), k1);
-    f.q2 = __fmul_rn(__ll2float_rn(e2), k2);
+    const float q0 = __fmul_rn(e0, k0);
+    f.q1 = __fmul_rn(e1, k1);
+    f.q2 = __fmul_rn(e2, k2);
     f.rho = __fadd_rn(__fadd_rn(q0, f.q1), f.q2);
     return f;
+}
+__device__ __forceinline__ Frag make_frag(long long e0, long long e1, long long e2, float k0, float k1, float k2) {
+    return edge_frag(__ll2float_rn(e0), __ll2float_rn(e1), __ll2float_rn(e2), k0, k1, k2);
 }
 
 // (rho, t) is in front of (rho2, t2): larger inverse depth, then lower index.

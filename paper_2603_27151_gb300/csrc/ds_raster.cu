@@ -172,14 +172,13 @@ __global__ void __launch_bounds__(kTilePix, DS_MINB_FWD)
                         }
                     }
                     if (!valid) continue;
-                    long long E[3];
-                    if (!tile_cover(sm, j, lx, ly, E)) continue;
+                    int t;
+                    Frag f;
+                    if (!tile_cover(sm, recs, vbase, j, h2, lx, ly, px, py, t, f)) continue;
                     if (mode == 1) {
                         ++cnt[0];
                         continue;
                     }
-                    const int t = h2.y;
-                    const Frag f = make_frag(E[0], E[1], E[2], sm.kk[j][0], sm.kk[j][1], sm.kk[j][2]);
 #pragma unroll
                     for (int q = 0; q < SG; ++q)
                         if (q < ns && (wt[q] < 0 || in_front(f.rho, t, wrho[q], wt[q]))) ++cnt[q];

@@ -31,15 +31,29 @@ constexpr unsigned kFullMask = 0xffffffffu;
 #define DS_MINB_TRAIN 5
 #endif
 
-// Per-tile staged set-up.  h0..h2 hold what the per-pixel coverage test reads
-// for every triangle; eo/kk are read only for covered fragments.
+// Per-tile staged set-up.  For the pixel at local offset (lx, ly) of the
+// tile, with the biased edge value E'(origin) = eb of the tile's first pixel
+// centre,
+//   s_i = A_i lx + B_i ly + (eb >> 8)   (int32; covered iff every s_i >= 0)
+//   E_i = r_i + 256 s_i,  r_i = (eb & 255) + bias_i   (the oriented value).
+// Inside the guard band |A|, |B| < 2^23 and lx, ly < 32, so |A lx + B ly| <
+// 2^29; eb >> 8 is clamped to +-2^30, which does not change the sign of s_i.
+// The E_i of a covered pixel are non-negative and add up to |2 area|: when
+// that is below 2^31 (triangles of up to 16,384 square pixels) they are
+// formed in int32, above (kBig) in int64, and where an edge value was clamped
+// (kHuge: more than 2^38, several screens away) from the set-up record.  All
+// give the same float: one rounding of the same integer.  The int64 to float
+// conversion runs on the FP64 pipe, at a small fraction of the rate of the
+// int32 one: with it for every fragment that pipe was busy 55% of a one-sample
+// forward (a threshold render of 200,000 triangles at 1080p).
 struct TileStage {
-    int4 h0[kChunk];         // A0, B0, thr0, A1
-    int4 h1[kChunk];         // B1, thr1, A2, B2
-    int4 h2[kChunk];         // thr2, triangle, rho bound (float bits), warp mask
-    long long eo[kChunk][3]; // oriented (unbiased) edge values at the tile's first pixel centre
-    float kk[kChunk][3];     // perspective factors k_i
+    int4 h0[kChunk];    // A0, B0, s0, A1
+    int4 h1[kChunk];    // B1, s1, A2, B2
+    int4 h2[kChunk];    // s2, triangle | flags, rho bound (float bits), warp mask
+    int4 h3[kChunk];    // r0, r1, r2, k0 (float bits): read for covered fragments only
+    float2 h4[kChunk];  // k1, k2
 };
+constexpr unsigned kBig = 1u << 31, kHuge = 1u << 30, kTriMask = DS_MAX_TRIANGLES - 1;
 
 struct WorkItem {
     int v, g, tx, ty;
@@ -74,30 +88,24 @@ __device__ __forceinline__ float rho_bound(uint32_t key, int DB) {
 }
 
 // Stage triangle t (set-up record in view base vbase) for the tile whose
-// first pixel is (ox, oy).  For a pixel at local offset (lx, ly) the biased
-// edge value is E'(origin) + 256 (A lx + B ly); it is >= 0 iff
-// A lx + B ly >= thr with thr = ceil(-E'(origin) / 256).  Inside the guard
-// band |A|, |B| < 2^23 and lx, ly < 32, so |A lx + B ly| < 2^29: thr is
-// clamped to +-2^30 and the test runs in int32.
+// first pixel is (ox, oy).
 //
 // h2.w receives a conservative mask of the tile's warps (bit w: the 32
 // pixels of threads 32w..32w+31, rows w*R .. w*R+R-1 with R = 32 / TW) whose
 // pixel centres the triangle may cover: for each edge the largest
-// A lx + B ly over the warp's rectangle (at a corner) must reach thr.
+// A lx + B ly over the warp's rectangle (at a corner) must reach -(eb >> 8).
 template <int TW>
 __device__ __forceinline__ void stage_triangle(TileStage& sm, int slot, const SetupRec* recs, size_t vbase,
                                                uint32_t key, uint32_t t, int DB, int ox, int oy) {
     const SetupRec r = load_rec(recs + vbase + t);
     const long long X0 = 256LL * ox + 128, Y0 = 256LL * oy + 128;
-    int thr[3];
+    int sv[3], rl[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         const long long eb = (long long)r.A[i] * X0 + (long long)r.B[i] * Y0 + r.C[i];
-        long long th = -(eb >> 8);
-        th = th < -(1LL << 30) ? -(1LL << 30) : (th > (1LL << 30) ? (1LL << 30) : th);
-        thr[i] = (int)th;
-        sm.eo[slot][i] = eb + ((r.bias >> i) & 1u);
-        sm.kk[slot][i] = r.k[i];
+        const long long th = eb >> 8;
+        sv[i] = th < -(1LL << 30) ? -(1 << 30) : (th > (1LL << 30) ? (1 << 30) : (int)th);
+        rl[i] = (int)(eb & 255) + (int)((r.bias >> i) & 1u);
     }
     constexpr int R = 32 / TW;   // rows per warp
     int wmask = 0;
@@ -108,26 +116,46 @@ __device__ __forceinline__ void stage_triangle(TileStage& sm, int slot, const Se
         for (int i = 0; i < 3; ++i) {
             const int mx = r.A[i] > 0 ? r.A[i] * (TW - 1) : 0;
             const int my = r.B[i] * (r.B[i] > 0 ? w * R + R - 1 : w * R);
-            may = may && (mx + my >= thr[i]);
+            may = may && (mx + my + sv[i] >= 0);
         }
         wmask |= may ? 1 << w : 0;
     }
-    sm.h0[slot] = make_int4(r.A[0], r.B[0], thr[0], r.A[1]);
-    sm.h1[slot] = make_int4(r.B[1], thr[1], r.A[2], r.B[2]);
-    sm.h2[slot] = make_int4(thr[2], (int)t, __float_as_int(rho_bound(key, DB)), wmask);
+    // |2 area| from two edge normals
+    if ((long long)r.A[0] * r.B[1] - (long long)r.A[1] * r.B[0] >= (1LL << 31)) t |= kBig;
+    if (max(sv[0], max(sv[1], sv[2])) == 1 << 30) t |= kHuge;
+    sm.h0[slot] = make_int4(r.A[0], r.B[0], sv[0], r.A[1]);
+    sm.h1[slot] = make_int4(r.B[1], sv[1], r.A[2], r.B[2]);
+    sm.h2[slot] = make_int4(sv[2], (int)t, __float_as_int(rho_bound(key, DB)), wmask);
+    sm.h3[slot] = make_int4(rl[0], rl[1], rl[2], __float_as_int(r.k[0]));
+    sm.h4[slot] = make_float2(r.k[1], r.k[2]);
 }
 
-// Coverage of local pixel (lx, ly) by staged triangle j; on success E gets
-// the exact oriented edge values (int64) at the pixel centre.
-__device__ __forceinline__ bool tile_cover(const TileStage& sm, int j, int lx, int ly, long long E[3]) {
-    const int4 h0 = sm.h0[j], h1 = sm.h1[j], h2 = sm.h2[j];
-    const int a0 = h0.x * lx + h0.y * ly;
-    const int a1 = h0.w * lx + h1.x * ly;
-    const int a2 = h1.z * lx + h1.w * ly;
-    if (((a0 - h0.z) | (a1 - h1.y) | (a2 - h2.x)) < 0) return false;
-    E[0] = sm.eo[j][0] + 256LL * a0;
-    E[1] = sm.eo[j][1] + 256LL * a1;
-    E[2] = sm.eo[j][2] + 256LL * a2;
+// Coverage of local pixel (lx, ly) -- pixel (px, py) of the view -- by staged
+// triangle j (h2: its h2 entry); on success its index and the pinned fragment
+// (the exact oriented edge values, rounded once).
+__device__ __forceinline__ bool tile_cover(const TileStage& sm, const SetupRec* __restrict__ recs, size_t vbase, int j,
+                                           int4 h2, int lx, int ly, int px, int py, int& t, Frag& f) {
+    const int4 h0 = sm.h0[j], h1 = sm.h1[j];
+    const int s0 = h0.x * lx + (h0.y * ly + h0.z);
+    const int s1 = h0.w * lx + (h1.x * ly + h1.y);
+    const int s2 = h1.z * lx + (h1.w * ly + h2.x);
+    if ((s0 | s1 | s2) < 0) return false;
+    const int4 h3 = sm.h3[j];
+    const float2 h4 = sm.h4[j];
+    t = h2.y & (int)kTriMask;
+    float e0, e1, e2;
+    if (!(h2.y & (int)(kBig | kHuge))) {
+        e0 = __int2float_rn(h3.x + (s0 << 8));
+        e1 = __int2float_rn(h3.y + (s1 << 8));
+        e2 = __int2float_rn(h3.z + (s2 << 8));
+    } else {
+        long long E[3] = {h3.x + 256LL * s0, h3.y + 256LL * s1, h3.z + 256LL * s2};
+        if (h2.y & (int)kHuge) cover_exact(load_rec(recs + vbase + t), px, py, E);
+        e0 = __ll2float_rn(E[0]);
+        e1 = __ll2float_rn(E[1]);
+        e2 = __ll2float_rn(E[2]);
+    }
+    f = edge_frag(e0, e1, e2, __int_as_float(h3.w), h4.x, h4.y);
     return true;
 }
 
@@ -172,10 +200,9 @@ __device__ __forceinline__ bool forward_walk(TileStage& sm, const SetupRec* __re
                     }
                 }
                 if (!valid) continue;
-                long long E[3];
-                if (!tile_cover(sm, j, lx, ly, E)) continue;
-                const int t = h2.y;
-                const Frag f = make_frag(E[0], E[1], E[2], sm.kk[j][0], sm.kk[j][1], sm.kk[j][2]);
+                int t;
+                Frag f;
+                if (!tile_cover(sm, recs, vbase, j, h2, lx, ly, px, py, t, f)) continue;
                 bool need = false;
 #pragma unroll
                 for (int q = 0; q < SG; ++q)
@@ -186,18 +213,21 @@ __device__ __forceinline__ bool forward_walk(TileStage& sm, const SetupRec* __re
                 const Cell cl = find_cell(s.N, b1, b2);
                 const float* aa = s.act_a + (size_t)t * s.V;
                 const float alpha = interp(__ldg(aa + cl.k0), __ldg(aa + cl.k1), __ldg(aa + cl.k2), cl.wa, cl.wb);
-                float tau[4] = {0.5f, 0.5f, 0.5f, 0.5f};
+                // alpha > tau on integers: tau = k 2^-24, and alpha 2^24 (exact)
+                // exceeds the integer k iff its ceiling does
+                const int ka = __float2int_ru(__fmul_rn(alpha, 0x1p24f));
+                int k[4] = {1 << 23, 1 << 23, 1 << 23, 1 << 23};   // tau = 1/2
                 if (stochastic) {
                     const uint4 w = philox4x32_10(make_uint4((uint32_t)px, (uint32_t)py, (uint32_t)t, (uint32_t)wi.g),
                                                   seed.x, seed.y);
-                    tau[0] = word_to_tau(w.x);
-                    tau[1] = word_to_tau(w.y);
-                    tau[2] = word_to_tau(w.z);
-                    tau[3] = word_to_tau(w.w);
+                    k[0] = (int)(w.x >> 8);
+                    k[1] = (int)(w.y >> 8);
+                    k[2] = (int)(w.z >> 8);
+                    k[3] = (int)(w.w >> 8);
                 }
 #pragma unroll
                 for (int q = 0; q < SG; ++q) {
-                    if (q < ns && alpha > tau[q] && (bt[q] < 0 || in_front(f.rho, t, brho[q], bt[q]))) {
+                    if (q < ns && ka > k[q] && (bt[q] < 0 || in_front(f.rho, t, brho[q], bt[q]))) {
                         bt[q] = t;
                         brho[q] = f.rho;
                         bb1[q] = b1;
@@ -429,12 +459,11 @@ __device__ __forceinline__ void score_walk(TileStage& sm, const SetupRec* __rest
                             break;
                         }
                     }
-                    const int t = h2.y;
+                    int t = 0;
+                    Frag f;
                     bool need = false;
                     float gw = 0.f, b1 = 0.f, b2 = 0.f;
-                    long long E[3];
-                    if (any_score && tile_cover(sm, j, lx, ly, E)) {
-                        const Frag f = make_frag(E[0], E[1], E[2], sm.kk[j][0], sm.kk[j][1], sm.kk[j][2]);
+                    if (any_score && tile_cover(sm, recs, vbase, j, h2, lx, ly, wi.tx * TW + lx, wi.ty * TH + ly, t, f)) {
 #pragma unroll
                         for (int q = 0; q < SG; ++q)
                             if (wsc[q] != 0.f && t != wt[q] && (wt[q] < 0 || in_front(f.rho, t, wrho[q], wt[q]))) {
