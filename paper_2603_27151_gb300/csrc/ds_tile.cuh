@@ -120,8 +120,8 @@ __device__ __forceinline__ void stage_triangle(TileStage& sm, int slot, const Se
         }
         wmask |= may ? 1 << w : 0;
     }
-    // |2 area| from two edge normals
-    if ((long long)r.A[0] * r.B[1] - (long long)r.A[1] * r.B[0] >= (1LL << 31)) t |= kBig;
+    // |2 area| from two edge normals (signed by the screen orientation)
+    if (llabs((long long)r.A[0] * r.B[1] - (long long)r.A[1] * r.B[0]) >= (1LL << 31)) t |= kBig;
     if (max(sv[0], max(sv[1], sv[2])) == 1 << 30) t |= kHuge;
     sm.h0[slot] = make_int4(r.A[0], r.B[0], sv[0], r.A[1]);
     sm.h1[slot] = make_int4(r.B[1], sv[1], r.A[2], r.B[2]);

@@ -28,7 +28,9 @@ def _scene():
     for _ in range(20):
         c = rng.uniform(0, 200, 2)
         tri.append([(*(c + rng.uniform(-40, 40, 2)), rng.uniform(0.9, 2.0)) for _ in range(3)])
+    tri += [[a, c, b] for a, b, c in tri[:9]]   # the other screen orientation, a little behind
     t = np.array(tri)
+    t[29:, :, 2] += 0.02
     cam = I.Camera(W, H, 64.0, 64.0, 0.0, 0.0, np.eye(3, dtype=np.float32), np.zeros(3, np.float32))
     verts = np.stack([t[..., 0] * t[..., 2] / 64.0, t[..., 1] * t[..., 2] / 64.0, t[..., 2]], -1).astype(np.float32)
     s = np.round(t[..., :2] * 256).astype(np.int64)
