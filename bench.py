@@ -2,7 +2,7 @@
 """Benchmark of the masked rasteriser's forward + backward pass.
 
 One step = the whole hot path on one batch: texture activation, triangle
-set-up, radix-sorted tile binning, the stochastically masked raster forward
+set-up, tile binning, the stochastically masked raster forward
 with texture decode, the fused L2 loss with its upstream gradients, and the
 backward (colour, opacity-score, interior and edge gradients).  Workload: the
 1080p large batch -- 100,000 triangles, 8x8 texel grids (N = 8, V = 45) of 8

@@ -14,7 +14,7 @@
  *  - Inputs are validated before any launch (sizes, counts, finiteness of
  *    cameras); a violation returns DS_ERR_INVALID_ARG and launches nothing.
  *  - The library owns its scratch memory (triangle set-up records, bin keys,
- *    sort buffers, activations); it grows it with cudaMalloc when a call
+ *    tile counts, activations); it grows it with cudaMalloc when a call
  *    needs more and frees it in ds_destroy.
  *
  * Notation (paper Sec. 3): T triangles; per-triangle mesh-colour grid with N
@@ -194,7 +194,7 @@ DS_API ds_status ds_levels_resample(const float* src, int32_t T, int32_t r_src, 
                                     int32_t r_dst, void* stream);
 
 /* Forward pass (Eq. 5; Algorithm A1 step 1) for n_views views of one soup:
- * sigmoid activation of the texture (Sec. 3.3), triangle set-up, radix-sorted
+ * sigmoid activation of the texture (Sec. 3.3), triangle set-up,
  * binning of triangles into tiles of 256 pixels (8x32, 16x16 or 32x8: a
  * launch parameter of the context, see ds_set_tuning), then per pixel and sample the
  * foremost covered fragment whose interpolated opacity exceeds its threshold
@@ -644,7 +644,7 @@ DS_API ds_status ds_server_destroy(ds_server* srv);
 
 /* Profiling (off by default; no paper counterpart: instrumentation).  While
  * enabled, every pipeline stage that a call on this context launches
- * (activate, setup, scan, emit, sort, ranges, raster_fwd, count, geom,
+ * (activate, setup, scan, emit, sort, raster_fwd, count, geom,
  * raster_bwd, edge_bwd, finish) is bracketed by two CUDA events recorded on the caller's stream.
  * ds_profile_read waits for those events and returns, for stage index
  * `stage` in [0, ds_profile_stages()), its name (static host string), the

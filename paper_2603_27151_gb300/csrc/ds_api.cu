@@ -1,6 +1,7 @@
 // ds_api.cu -- the C ABI declared in include/diffsoup.h: contexts, soups,
 // scratch management and the launch sequence of the forward and backward
 // passes.  Host code only.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -84,7 +85,6 @@ struct Plan {
     int soup = -1;
     std::vector<ds_camera> cams;
     int DB = 0;
-    int res = 0;
     uint32_t kcap = 0;
     int n_tiles = 0;
 };
@@ -109,13 +109,12 @@ struct ds_ctx {
     int device = 0;
     std::mutex mu;
     std::vector<Soup> soups;
-    DevBuf recs, counts, offs, tbox, zkeys, keys[2], vals[2], hist, hist_scan, ranges, scanbuf, misc, geom;
+    DevBuf recs, tbox, zkeys, keys[2], vals[2], tcount, tcursor, tsums, ranges, misc, geom;
     DevBuf acc_tex, acc_verts;   // FP64 gradient accumulators of the backward
     DevBuf shade_part;           // per-CTA partials of the shading parameter gradients
     DevBuf plan_dev;             // device copy of an adaptive-control plan
-    ds::ScanScratch scan;
-    int64_t scan_cap = 0;
     uint32_t* h_word = nullptr;   // pinned host words
+    cudaEvent_t k_event = nullptr;   // the pair count has reached h_word
     Plan plan;
     ds_tuning tune{16, -1, 0, 256};   // tile shape, depth bits, grid, staging chunk
     int32_t shade_path = DS_SHADE_TENSOR_CORES;   // kernel of ds_shade_forward
@@ -134,7 +133,7 @@ struct ds_ctx {
     double prof_ms[ds::kNumStages] = {0};
     long long prof_n[ds::kNumStages] = {0};
 
-    // misc layout
+    // misc layout (work counters: 0 forward, 1 and 4 counts, 2 backward, 3 edges)
     int* d_status() const { return misc.as<int>(); }
     int* d_counter() const { return misc.as<int>() + 4; }
     uint32_t* d_K() const { return reinterpret_cast<uint32_t*>(misc.as<int>() + 12); }
@@ -142,6 +141,14 @@ struct ds_ctx {
 };
 
 namespace {
+
+constexpr int kCounters = 5;
+
+// Pairs that every list buffer holds.
+uint32_t pair_capacity(const ds_ctx* c) {
+    size_t n = std::min(std::min(c->keys[0].cap, c->keys[1].cap), std::min(c->vals[0].cap, c->vals[1].cap)) / 4;
+    return (uint32_t)std::min<size_t>(n, 0xffffffffu);
+}
 
 struct DeviceGuard {
     int prev = -1;
@@ -204,26 +211,6 @@ ds_status prof_flush(ds_ctx* c) {
         c->prof_pool.push_back(r.b);
     }
     c->prof_pending.clear();
-    return DS_OK;
-}
-
-ds_status ensure_scan(ds_ctx* c, int64_t n) {
-    if (n <= c->scan_cap && c->scanbuf.p) return DS_OK;
-    int64_t sizes[6] = {0};
-    const int lv = ds::scan_levels(n, sizes);
-    int64_t total = 0;
-    for (int i = 0; i < lv; ++i) total += 2 * sizes[i];
-    DS_TRY(c->scanbuf.ensure(sizeof(uint32_t) * (size_t)(total + 1), "scan scratch"));
-    uint32_t* p = c->scanbuf.as<uint32_t>();
-    c->scan.levels = lv;
-    for (int i = 0; i < lv; ++i) {
-        c->scan.level_n[i] = sizes[i];
-        c->scan.level[i] = p;
-        p += sizes[i];
-        c->scan.level_out[i] = p;
-        p += sizes[i];
-    }
-    c->scan_cap = n;
     return DS_OK;
 }
 
@@ -363,12 +350,12 @@ ds_status prepare(ds_ctx* c, int32_t plan_soup, Soup* const* soups, const ds_cam
     const int n_tiles = total_tiles(vt);
     c->plan.valid = false;
     DS_TRY(c->recs.ensure(sizeof(ds::SetupRec) * nvt, "set-up records"));
-    DS_TRY(c->counts.ensure(4 * nvt, "tile counts"));
-    DS_TRY(c->offs.ensure(4 * nvt, "tile offsets"));
     DS_TRY(c->tbox.ensure(16 * nvt, "tile boxes"));
     DS_TRY(c->zkeys.ensure(4 * nvt, "depth keys"));
     DS_TRY(c->ranges.ensure(8 * (size_t)n_tiles, "tile ranges"));
-    DS_TRY(ensure_scan(c, (int64_t)nvt));
+    DS_TRY(c->tcount.ensure(4 * (size_t)n_tiles, "tile counts"));
+    DS_TRY(c->tcursor.ensure(4 * (size_t)n_tiles, "tile cursors"));
+    DS_TRY(c->tsums.ensure(4 * ((size_t)n_tiles / ds::kScanBlock + 1), "tile scan sums"));
 
     for (int v = 0; v < vt.n; ++v) {
         Soup& s = *soups[v];
@@ -384,51 +371,53 @@ ds_status prepare(ds_ctx* c, int32_t plan_soup, Soup* const* soups, const ds_cam
     }
     {
         StageScope p(c, ds::kStSetup, st);
-        DS_TRY_CUDA(ds::launch_setup(vt, c->recs.as<ds::SetupRec>(), c->counts.as<uint32_t>(), c->tbox.as<int4>(),
-                                     c->zkeys.as<uint32_t>(), st));
+        DS_TRY_CUDA(ds::launch_setup(vt, n_tiles, c->recs.as<ds::SetupRec>(), c->tcount.as<uint32_t>(),
+                                     c->tbox.as<int4>(), c->zkeys.as<uint32_t>(), st));
     }
-    {
+    uint32_t cap = pair_capacity(c);
+    const bool wait = sync || cap == 0;
+    const int tile_bits = bits_for((uint32_t)n_tiles);
+    const int DB = std::min(c->tune.depth_bits >= 0 ? c->tune.depth_bits : 16, 32 - tile_bits);
+    auto offsets = [&](uint32_t limit) {
         StageScope p(c, ds::kStScan, st);
-        DS_TRY_CUDA(ds::scan_exclusive(c->counts.as<uint32_t>(), c->offs.as<uint32_t>(), (int64_t)nvt, c->d_K(), c->scan, st));
-    }
-
-    uint32_t kcap = (uint32_t)(c->keys[0].cap / 4);
-    if (sync || kcap == 0) {
+        return ds::launch_tile_offsets(c->tcount.as<uint32_t>(), n_tiles, limit, c->tsums.as<uint32_t>(),
+                                       c->ranges.as<uint2>(), c->tcursor.as<uint32_t>(), c->d_K(), c->d_counter(),
+                                       kCounters, st);
+    };
+    auto lists = [&](uint32_t limit, int* status) {
+        cudaError_t e = cudaSuccess;
+        {
+            StageScope p(c, ds::kStEmit, st);
+            e = ds::launch_emit(vt, c->recs.as<ds::SetupRec>(), c->tbox.as<int4>(), c->zkeys.as<uint32_t>(), DB,
+                                c->tcursor.as<uint32_t>(), c->keys[0].as<uint32_t>(), c->vals[0].as<uint32_t>(), limit,
+                                status, st);
+        }
+        if (e != cudaSuccess || DB <= 0) return e;
+        StageScope p(c, ds::kStSort, st);
+        return ds::launch_tile_sort(c->ranges.as<uint2>(), n_tiles, DB, c->keys[0].as<uint32_t>(),
+                                    c->vals[0].as<uint32_t>(), c->keys[1].as<uint32_t>(), c->vals[1].as<uint32_t>(), st);
+    };
+    DS_TRY_CUDA(offsets(cap));
+    // With a host wait for the number of pairs: the lists are built with the
+    // buffers there are while the number travels, and built again if they
+    // turn out to be too small.
+    if (wait) {
         DS_TRY_CUDA(cudaMemcpyAsync(c->h_word, c->d_K(), 4, cudaMemcpyDeviceToHost, st));
-        DS_TRY_CUDA(cudaStreamSynchronize(st));
+        DS_TRY_CUDA(cudaEventRecord(c->k_event, st));
+    }
+    if (cap > 0) DS_TRY_CUDA(lists(cap, wait ? nullptr : c->d_status()));
+    if (wait) {
+        DS_TRY_CUDA(cudaEventSynchronize(c->k_event));
         const uint32_t K = *c->h_word;
-        if ((size_t)K * 4 > c->keys[0].cap || !c->keys[0].p) {
+        if (K > cap || cap == 0) {
             for (int b = 0; b < 2; ++b) {
                 DS_TRY(c->keys[b].ensure(4 * (size_t)(K > 0 ? K : 1), "bin keys"));
                 DS_TRY(c->vals[b].ensure(4 * (size_t)(K > 0 ? K : 1), "bin values"));
             }
+            DS_TRY_CUDA(offsets(pair_capacity(c)));
+            DS_TRY_CUDA(lists(pair_capacity(c), nullptr));
         }
-        kcap = K;
-    }
-    const uint32_t nblk = (kcap + ds::kSortBlock - 1) / ds::kSortBlock;
-    DS_TRY(c->hist.ensure(4 * 256 * (size_t)(nblk > 0 ? nblk : 1), "radix histogram"));
-    DS_TRY(c->hist_scan.ensure(4 * 256 * (size_t)(nblk > 0 ? nblk : 1), "radix offsets"));
-    DS_TRY(ensure_scan(c, (int64_t)256 * (nblk > 0 ? nblk : 1)));
-
-    const int tile_bits = bits_for((uint32_t)n_tiles);
-    const int DB = std::min(c->tune.depth_bits >= 0 ? c->tune.depth_bits : 16, 32 - tile_bits);
-    {
-        StageScope p(c, ds::kStEmit, st);
-        DS_TRY_CUDA(ds::launch_emit(vt, c->recs.as<ds::SetupRec>(), c->counts.as<uint32_t>(), c->offs.as<uint32_t>(),
-                                    c->tbox.as<int4>(), c->zkeys.as<uint32_t>(), DB, c->keys[0].as<uint32_t>(),
-                                    c->vals[0].as<uint32_t>(), kcap, c->d_status(), st));
-    }
-    cudaError_t se = cudaSuccess;
-    StageScope* sort_scope = new StageScope(c, ds::kStSort, st);
-    const int res = ds::radix_sort_pairs(c->keys[0].as<uint32_t>(), c->vals[0].as<uint32_t>(), c->keys[1].as<uint32_t>(),
-                                         c->vals[1].as<uint32_t>(), c->d_K(), kcap, tile_bits + DB,
-                                         c->hist.as<uint32_t>(), c->hist_scan.as<uint32_t>(), c->scan, st, &se);
-    delete sort_scope;
-    DS_TRY_CUDA(se);
-    {
-        StageScope p(c, ds::kStRanges, st);
-        DS_TRY_CUDA(cudaMemsetAsync(c->ranges.p, 0, 8 * (size_t)n_tiles, st));
-        DS_TRY_CUDA(ds::launch_tile_ranges(c->keys[res].as<uint32_t>(), c->d_K(), kcap, DB, c->ranges.as<uint2>(), st));
+        cap = K;
     }
 
     c->plan.valid = true;
@@ -440,8 +429,7 @@ ds_status prepare(ds_ctx* c, int32_t plan_soup, Soup* const* soups, const ds_cam
     else
         c->plan.cams.clear();
     c->plan.DB = DB;
-    c->plan.res = res;
-    c->plan.kcap = kcap;
+    c->plan.kcap = cap;
     c->plan.n_tiles = n_tiles;
     return DS_OK;
 }
@@ -485,14 +473,22 @@ ds_status ds_create(ds_ctx** out, int32_t device) {
     }
     c->device = device;
     DeviceGuard g(device);
+    if (cudaEventCreateWithFlags(&c->k_event, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        delete[] c->vt;
+        delete c;
+        return fail(DS_ERR_CUDA, "cudaEventCreate failed");
+    }
     if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_word), 64, cudaHostAllocDefault) != cudaSuccess) {
         cudaGetLastError();
+        cudaEventDestroy(c->k_event);
         delete[] c->vt;
         delete c;
         return fail(DS_ERR_CUDA, "cudaHostAlloc failed");
     }
     if (c->misc.ensure(256, "context words") != DS_OK) {
         cudaFreeHost(c->h_word);
+        cudaEventDestroy(c->k_event);
         delete[] c->vt;
         delete c;
         return DS_ERR_OOM;
@@ -510,11 +506,11 @@ void ds_destroy(ds_ctx* c) {
         if (s.own) cudaFree(s.own);
         if (s.act) cudaFree(s.act);
     }
-    DevBuf* bufs[] = {&c->recs,  &c->counts,  &c->offs,      &c->tbox,   &c->zkeys,   &c->keys[0], &c->keys[1],
-                      &c->vals[0], &c->vals[1], &c->hist, &c->hist_scan, &c->ranges, &c->scanbuf, &c->misc,
-                      &c->geom, &c->acc_tex, &c->acc_verts, &c->shade_part, &c->plan_dev};
+    DevBuf* bufs[] = {&c->recs, &c->tbox, &c->zkeys, &c->keys[0], &c->keys[1], &c->vals[0], &c->vals[1],
+                      &c->tcount, &c->tcursor, &c->tsums, &c->ranges, &c->misc, &c->geom, &c->acc_tex, &c->acc_verts, &c->shade_part, &c->plan_dev};
     for (DevBuf* b : bufs) b->release();
     if (c->h_word) cudaFreeHost(c->h_word);
+    if (c->k_event) cudaEventDestroy(c->k_event);
     for (auto& r : c->prof_pending) {
         cudaEventDestroy(r.a);
         cudaEventDestroy(r.b);
@@ -701,18 +697,16 @@ ds_status forward_impl(ds_ctx* c, int32_t soup_id, Soup& s, const ds_camera* hos
     const int grid = tile_grid(c, vt);
     {
         StageScope p(c, ds::kStRasterFwd, st);
-        DS_TRY_CUDA(cudaMemsetAsync(c->d_counter(), 0, 4, st));
-        DS_TRY_CUDA(ds::launch_raster_fwd(vt, sd, c->recs.as<ds::SetupRec>(), c->keys[c->plan.res].as<uint32_t>(),
-                                          c->vals[c->plan.res].as<uint32_t>(), c->ranges.as<uint2>(), c->plan.DB,
+        DS_TRY_CUDA(ds::launch_raster_fwd(vt, sd, c->recs.as<ds::SetupRec>(), c->keys[0].as<uint32_t>(),
+                                          c->vals[0].as<uint32_t>(), c->ranges.as<uint2>(), c->plan.DB,
                                           mode & 0xffu, b, c->d_counter(), grid, st));
     }
     bool want_front = false;
     for (int v = 0; v < vt.n; ++v) want_front = want_front || out[v].n_front;
     if (want_front) {
         StageScope p(c, ds::kStCount, st);
-        DS_TRY_CUDA(cudaMemsetAsync(c->d_counter() + 1, 0, 4, st));
-        DS_TRY_CUDA(ds::launch_raster_count(vt, sd, c->recs.as<ds::SetupRec>(), c->keys[c->plan.res].as<uint32_t>(),
-                                            c->vals[c->plan.res].as<uint32_t>(), c->ranges.as<uint2>(), c->plan.DB, 0,
+        DS_TRY_CUDA(ds::launch_raster_count(vt, sd, c->recs.as<ds::SetupRec>(), c->keys[0].as<uint32_t>(),
+                                            c->vals[0].as<uint32_t>(), c->ranges.as<uint2>(), c->plan.DB, 0,
                                             nullptr, c->d_counter() + 1, grid, st));
     }
     return DS_OK;
@@ -747,6 +741,8 @@ ds_status backward_impl(ds_ctx* c, Soup& s, uint32_t grad_flags, float* grad_ver
     const bool want_tex = (grad_tex || tex_adam) && (gflags & (DS_G_TEX | DS_G_SCORE));
     const bool want_verts = grad_verts && (gflags & (DS_G_INTERIOR | DS_G_EDGE));
     const bool overwrite = (grad_flags & DS_OVERWRITE) != 0;
+    // the plan's scan has cleared the work counters; a reused plan's are used up
+    if (!fused) DS_TRY_CUDA(cudaMemsetAsync(c->d_counter() + 2, 0, 8, st));
     double* acc_tex = nullptr;
     double* acc_verts = nullptr;
     if (want_tex) {
@@ -766,39 +762,34 @@ ds_status backward_impl(ds_ctx* c, Soup& s, uint32_t grad_flags, float* grad_ver
         // split schedule: forward with the loss epilogue, then the backward
         {
             StageScope p(c, ds::kStRasterFwd, st);
-            DS_TRY_CUDA(cudaMemsetAsync(c->d_counter(), 0, 4, st));
             DS_TRY_CUDA(ds::launch_raster_fwd(vt, sd, c->recs.as<ds::SetupRec>(),
-                                              c->keys[c->plan.res].as<uint32_t>(), c->vals[c->plan.res].as<uint32_t>(),
+                                              c->keys[0].as<uint32_t>(), c->vals[0].as<uint32_t>(),
                                               c->ranges.as<uint2>(), c->plan.DB, fused->mode & 0xffu, fused->bg,
                                               c->d_counter(), grid, st, true, fused->scale, fused->loss));
         }
         if (want_tex || (want_verts && (gflags & DS_G_INTERIOR))) {
             StageScope p(c, ds::kStRasterBwd, st);
-            DS_TRY_CUDA(cudaMemsetAsync(c->d_counter() + 2, 0, 4, st));
             DS_TRY_CUDA(ds::launch_raster_bwd(vt, sd, c->recs.as<ds::SetupRec>(),
-                                              c->keys[c->plan.res].as<uint32_t>(), c->vals[c->plan.res].as<uint32_t>(),
+                                              c->keys[0].as<uint32_t>(), c->vals[0].as<uint32_t>(),
                                               c->ranges.as<uint2>(), c->plan.DB, gflags, c->geom.as<ds::GeomRec>(),
                                               acc_tex, acc_verts, c->d_counter() + 2, grid, st));
         }
     } else if (fused) {
         StageScope p(c, ds::kStTrain, st);
-        DS_TRY_CUDA(cudaMemsetAsync(c->d_counter() + 2, 0, 4, st));
-        DS_TRY_CUDA(ds::launch_raster_train(vt, sd, c->recs.as<ds::SetupRec>(), c->keys[c->plan.res].as<uint32_t>(),
-                                            c->vals[c->plan.res].as<uint32_t>(), c->ranges.as<uint2>(), c->plan.DB,
+        DS_TRY_CUDA(ds::launch_raster_train(vt, sd, c->recs.as<ds::SetupRec>(), c->keys[0].as<uint32_t>(),
+                                            c->vals[0].as<uint32_t>(), c->ranges.as<uint2>(), c->plan.DB,
                                             fused->mode & 0xffu, fused->bg, fused->scale, fused->loss, gflags,
                                             c->geom.as<ds::GeomRec>(), acc_tex, acc_verts, c->d_counter() + 2, grid,
                                             st));
     } else if (want_tex || (want_verts && (gflags & DS_G_INTERIOR))) {
         StageScope p(c, ds::kStRasterBwd, st);
-        DS_TRY_CUDA(cudaMemsetAsync(c->d_counter() + 2, 0, 4, st));
-        DS_TRY_CUDA(ds::launch_raster_bwd(vt, sd, c->recs.as<ds::SetupRec>(), c->keys[c->plan.res].as<uint32_t>(),
-                                          c->vals[c->plan.res].as<uint32_t>(), c->ranges.as<uint2>(), c->plan.DB,
+        DS_TRY_CUDA(ds::launch_raster_bwd(vt, sd, c->recs.as<ds::SetupRec>(), c->keys[0].as<uint32_t>(),
+                                          c->vals[0].as<uint32_t>(), c->ranges.as<uint2>(), c->plan.DB,
                                           gflags, c->geom.as<ds::GeomRec>(), acc_tex, acc_verts, c->d_counter() + 2,
                                           grid, st));
     }
     if (want_verts && (gflags & DS_G_EDGE)) {
         StageScope p(c, ds::kStEdgeBwd, st);
-        DS_TRY_CUDA(cudaMemsetAsync(c->d_counter() + 3, 0, 4, st));
         ds::ViewTable& ve = c->vt[1];
         retile(vt, kEdgeTileW, ve);
         DS_TRY_CUDA(ds::launch_edge_bwd(ve, sd, c->recs.as<ds::SetupRec>(), c->geom.as<ds::GeomRec>(), acc_verts,
@@ -922,18 +913,16 @@ ds_status ds_raster_forward_multi(ds_ctx* c, const int32_t* soup_ids, const ds_c
     const int grid = tile_grid(c, vt);
     {
         StageScope p(c, ds::kStRasterFwd, st);
-        DS_TRY_CUDA(cudaMemsetAsync(c->d_counter(), 0, 4, st));
-        DS_TRY_CUDA(ds::launch_raster_fwd(vt, sd, c->recs.as<ds::SetupRec>(), c->keys[c->plan.res].as<uint32_t>(),
-                                          c->vals[c->plan.res].as<uint32_t>(), c->ranges.as<uint2>(), c->plan.DB,
+        DS_TRY_CUDA(ds::launch_raster_fwd(vt, sd, c->recs.as<ds::SetupRec>(), c->keys[0].as<uint32_t>(),
+                                          c->vals[0].as<uint32_t>(), c->ranges.as<uint2>(), c->plan.DB,
                                           mode & 0xffu, b, c->d_counter(), grid, st, false, 0.f, nullptr, true));
     }
     bool want_front = false;
     for (int v = 0; v < vt.n; ++v) want_front = want_front || out[v].n_front;
     if (want_front) {
         StageScope p(c, ds::kStCount, st);
-        DS_TRY_CUDA(cudaMemsetAsync(c->d_counter() + 1, 0, 4, st));
-        DS_TRY_CUDA(ds::launch_raster_count(vt, sd, c->recs.as<ds::SetupRec>(), c->keys[c->plan.res].as<uint32_t>(),
-                                            c->vals[c->plan.res].as<uint32_t>(), c->ranges.as<uint2>(), c->plan.DB, 0,
+        DS_TRY_CUDA(ds::launch_raster_count(vt, sd, c->recs.as<ds::SetupRec>(), c->keys[0].as<uint32_t>(),
+                                            c->vals[0].as<uint32_t>(), c->ranges.as<uint2>(), c->plan.DB, 0,
                                             nullptr, c->d_counter() + 1, grid, st));
     }
     return DS_OK;
@@ -1034,10 +1023,6 @@ ds_status ds_reserve(ds_ctx* c, int64_t pairs) {
         DS_TRY(c->keys[b].ensure(4 * K, "bin keys"));
         DS_TRY(c->vals[b].ensure(4 * K, "bin values"));
     }
-    const size_t nblk = (K + ds::kSortBlock - 1) / ds::kSortBlock;
-    DS_TRY(c->hist.ensure(4 * 256 * nblk, "radix histogram"));
-    DS_TRY(c->hist_scan.ensure(4 * 256 * nblk, "radix offsets"));
-    DS_TRY(ensure_scan(c, (int64_t)(256 * nblk)));
     return DS_OK;
 }
 
@@ -1057,9 +1042,8 @@ ds_status ds_fragment_count(ds_ctx* c, int32_t soup_id, const ds_camera* cams, i
     const ds::SoupDev sd = soup_dev(*s);
     const int grid = tile_grid(c, vt);
     DS_TRY_CUDA(cudaMemsetAsync(c->d_total(), 0, 8, st));
-    DS_TRY_CUDA(cudaMemsetAsync(c->d_counter() + 4, 0, 4, st));
-    DS_TRY_CUDA(ds::launch_raster_count(vt, sd, c->recs.as<ds::SetupRec>(), c->keys[c->plan.res].as<uint32_t>(),
-                                        c->vals[c->plan.res].as<uint32_t>(), c->ranges.as<uint2>(), c->plan.DB, 1,
+    DS_TRY_CUDA(ds::launch_raster_count(vt, sd, c->recs.as<ds::SetupRec>(), c->keys[0].as<uint32_t>(),
+                                        c->vals[0].as<uint32_t>(), c->ranges.as<uint2>(), c->plan.DB, 1,
                                         c->d_total(), c->d_counter() + 4, grid, st));
     DS_TRY_CUDA(cudaMemcpyAsync(c->h_word, c->d_total(), 8, cudaMemcpyDeviceToHost, st));
     DS_TRY_CUDA(cudaStreamSynchronize(st));

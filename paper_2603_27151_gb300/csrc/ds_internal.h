@@ -13,7 +13,7 @@ namespace ds {
 
 // Pipeline stages timed by the optional profiler (ds_profile_*).
 enum Stage {
-    kStActivate, kStSetup, kStScan, kStEmit, kStSort, kStRanges,
+    kStActivate, kStSetup, kStScan, kStEmit, kStSort,
     kStRasterFwd, kStCount, kStGeom, kStRasterBwd, kStEdgeBwd, kStFinish, kStTrain, kNumStages
 };
 extern const char* const kStageNames[kNumStages];
@@ -36,34 +36,9 @@ void build_table(ViewTable& vt, const ds_tuning& tu, const ds_camera* cams, cons
 void note_launches(int n);
 long long launches_total();
 
-// Scratch for the multi-level exclusive scan (one sum buffer per level).
-struct ScanScratch {
-    uint32_t* level[6] = {nullptr};
-    uint32_t* level_out[6] = {nullptr};
-    int64_t level_n[6] = {0};
-    int levels = 0;
-};
+constexpr int kScanBlock = 4096;    // tiles per block of the tile scan (1024 threads x 4)
 
-constexpr int kScanBlock = 4096;    // items per scan block (1024 threads x 4)
-constexpr int kSortBlock = 4096;    // keys per radix-sort block (256 threads x 16)
-
-// Number of level buffers (and their sizes) needed to scan n items.
-int scan_levels(int64_t n, int64_t sizes[6]);
-
-// out[i] = sum_{j<i} in[j]; *total = sum of all (device).  in != out.
-cudaError_t scan_exclusive(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* total,
-                           const ScanScratch& sc, cudaStream_t st);
-
-// Stable LSD radix sort of (key, value) pairs on bits [0, nbits) with 8-bit
-// digits.  The pair count is read on the device from *count; kcap bounds it
-// (grid size).  Buffers ping-pong between (k0, v0) and (k1, v1); returns the
-// index (0 or 1) of the pair holding the result.
-int radix_sort_pairs(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1,
-                     const uint32_t* count, uint32_t kcap, int nbits, uint32_t* hist,
-                     uint32_t* hist_scan, const ScanScratch& sc, cudaStream_t st,
-                     cudaError_t* err);
-
-// ---- set-up and binning (ds_setup.cu)
+// ---- activation (ds_activate.cu), set-up and binning (ds_bin.cu)
 cudaError_t launch_activate(const SoupDev& s, cudaStream_t st);
 // The views' soups (ViewDesc s_*, rec_base): one soup for every view, or
 // soups[v] for view v (records of the views concatenated in view order);
@@ -71,15 +46,25 @@ cudaError_t launch_activate(const SoupDev& s, cudaStream_t st);
 void set_view_soups(ViewTable& vt, const SoupDev& s);
 void set_view_soups(ViewTable& vt, const SoupDev* const* soups);
 long long view_records(const ViewTable& vt);
-// One set-up record (and tile count, tile box, depth key) per (view,
-// triangle of the view's soup), at rec_base + triangle.
-cudaError_t launch_setup(const ViewTable& vt, SetupRec* recs, uint32_t* counts, int4* tbox, uint32_t* zkeys,
-                         cudaStream_t st);
-cudaError_t launch_emit(const ViewTable& vt, const SetupRec* recs, const uint32_t* counts, const uint32_t* offs,
-                        const int4* tbox, const uint32_t* zkeys, int DB, uint32_t* keys, uint32_t* vals,
-                        uint32_t cap, int* status, cudaStream_t st);
-cudaError_t launch_tile_ranges(const uint32_t* keys, const uint32_t* count, uint32_t kcap, int DB,
-                               uint2* ranges, cudaStream_t st);
+// One set-up record (and tile box, depth key) per (view, triangle of the
+// view's soup), at rec_base + triangle; tile_count [n_tiles]: the triangles
+// of every tile.
+cudaError_t launch_setup(const ViewTable& vt, int n_tiles, SetupRec* recs, uint32_t* tile_count, int4* tbox,
+                         uint32_t* zkeys, cudaStream_t st);
+// Scan of the counts: every tile's list range (cut at cap pairs), its cursor
+// for the emission, the number of pairs *total; sets counters[0 ..
+// n_counters-1] to zero.  block_sum: scratch, one word per kScanBlock tiles.
+cudaError_t launch_tile_offsets(const uint32_t* count, int n_tiles, uint32_t cap, uint32_t* block_sum, uint2* ranges,
+                                uint32_t* cursor, uint32_t* total, int* counters, int n_counters, cudaStream_t st);
+// Every (tile, triangle) pair into its tile's list: vals the triangles, keys
+// the DB depth bits (not written when DB = 0).  Beyond cap: bit 0 of *status
+// (if status is not NULL).
+cudaError_t launch_emit(const ViewTable& vt, const SetupRec* recs, const int4* tbox, const uint32_t* zkeys, int DB,
+                        uint32_t* cursor, uint32_t* keys, uint32_t* vals, uint32_t cap, int* status, cudaStream_t st);
+// The lists front to back (nothing to do when DB = 0); k1, v1: scratch of the
+// lists' size.
+cudaError_t launch_tile_sort(const uint2* ranges, int n_tiles, int DB, uint32_t* k0, uint32_t* v0, uint32_t* k1,
+                             uint32_t* v1, cudaStream_t st);
 
 // ---- forward rasteriser (ds_raster.cu)
 // multi: every view reads its own soup (ViewDesc s_*, rec_base) instead of s

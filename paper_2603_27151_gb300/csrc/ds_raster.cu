@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(kTilePix, DS_MINB_FWD)
             const int n = (int)min((uint32_t)vt.chunk, rg.y - c0);
             __syncthreads();
             if (tid < n)
-                stage_triangle<TW>(sm, tid, recs, vbase, keys[c0 + tid], vals[c0 + tid], DB, wi.tx * TW, wi.ty * TH);
+                stage_triangle<TW>(sm, tid, recs, vbase, DB > 0 ? keys[c0 + tid] : 0u, vals[c0 + tid], DB, wi.tx * TW, wi.ty * TH);
             __syncthreads();
             if (!warp_done) {
                 for (int j = 0; j < n; ++j) {
@@ -238,7 +238,7 @@ cudaError_t launch_raster_count(const ViewTable& vt, const SoupDev& s, const Set
     return cudaGetLastError();
 }
 
-const char* const kStageNames[kNumStages] = {"activate", "setup", "scan", "emit", "sort", "ranges",
+const char* const kStageNames[kNumStages] = {"activate", "setup", "scan", "emit", "sort",
                                              "raster_fwd", "count", "geom", "raster_bwd", "edge_bwd",
                                              "finish", "train"};
 

@@ -18,7 +18,6 @@ constexpr long long kMaxViewTris = 1LL << 16;    // n_views * T
 constexpr long long kMaxPairs = 1LL << 19;       // (tile, triangle) pairs after binning
 constexpr int kTileEdge = 16;                    // tiles of 16x16 pixels
 constexpr long long kMaxTiles = 1LL << 16;       // 16x16 tiles over all views
-constexpr long long kMaxSortBlocks = kMaxPairs / ds::kSortBlock;
 
 constexpr size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
@@ -26,19 +25,16 @@ constexpr size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 constexpr size_t kOffAct = 0;
 constexpr size_t kOffActA = align256(kOffAct + 4 * kMaxTexFloats);
 constexpr size_t kOffRecs = align256(kOffActA + 4 * (kMaxTexFloats / 2));
-constexpr size_t kOffCounts = align256(kOffRecs + sizeof(ds::SetupRec) * kMaxViewTris);
-constexpr size_t kOffOffs = align256(kOffCounts + 4 * kMaxViewTris);
-constexpr size_t kOffBox = align256(kOffOffs + 4 * kMaxViewTris);
+constexpr size_t kOffBox = align256(kOffRecs + sizeof(ds::SetupRec) * kMaxViewTris);
 constexpr size_t kOffZkeys = align256(kOffBox + 16 * kMaxViewTris);
 constexpr size_t kOffKeys0 = align256(kOffZkeys + 4 * kMaxViewTris);
 constexpr size_t kOffVals0 = align256(kOffKeys0 + 4 * kMaxPairs);
 constexpr size_t kOffKeys1 = align256(kOffVals0 + 4 * kMaxPairs);
 constexpr size_t kOffVals1 = align256(kOffKeys1 + 4 * kMaxPairs);
-constexpr size_t kOffHist = align256(kOffVals1 + 4 * kMaxPairs);
-constexpr size_t kOffHistScan = align256(kOffHist + 4 * 256 * kMaxSortBlocks);
-constexpr size_t kOffScan = align256(kOffHistScan + 4 * 256 * kMaxSortBlocks);
-constexpr size_t kScanWords = 2 * 64;            // level buffers: inputs up to 2^18 items
-constexpr size_t kOffRanges = align256(kOffScan + 4 * kScanWords);
+constexpr size_t kOffCount = align256(kOffVals1 + 4 * kMaxPairs);
+constexpr size_t kOffCursor = align256(kOffCount + 4 * kMaxTiles);
+constexpr size_t kOffSums = align256(kOffCursor + 4 * kMaxTiles);
+constexpr size_t kOffRanges = align256(kOffSums + 4 * (kMaxTiles / ds::kScanBlock + 1));
 constexpr size_t kOffMisc = align256(kOffRanges + 8 * kMaxTiles);
 constexpr size_t kStaticBytes = align256(kOffMisc + 256);   // about 21 MiB
 
@@ -143,32 +139,18 @@ extern "C" DS_API ds_status ds_raster_forward_noalloc(const float* verts, const 
     sd.C = C;
     sd.V = V;
     auto* recs = reinterpret_cast<ds::SetupRec*>(base + kOffRecs);
-    auto* counts = reinterpret_cast<uint32_t*>(base + kOffCounts);
-    auto* offs = reinterpret_cast<uint32_t*>(base + kOffOffs);
     auto* tbox = reinterpret_cast<int4*>(base + kOffBox);
     auto* zkeys = reinterpret_cast<uint32_t*>(base + kOffZkeys);
     uint32_t* keys[2] = {reinterpret_cast<uint32_t*>(base + kOffKeys0), reinterpret_cast<uint32_t*>(base + kOffKeys1)};
     uint32_t* vals[2] = {reinterpret_cast<uint32_t*>(base + kOffVals0), reinterpret_cast<uint32_t*>(base + kOffVals1)};
-    auto* hist = reinterpret_cast<uint32_t*>(base + kOffHist);
-    auto* hist_scan = reinterpret_cast<uint32_t*>(base + kOffHistScan);
+    auto* tcount = reinterpret_cast<uint32_t*>(base + kOffCount);
+    auto* tcursor = reinterpret_cast<uint32_t*>(base + kOffCursor);
+    auto* tsums = reinterpret_cast<uint32_t*>(base + kOffSums);
     auto* ranges = reinterpret_cast<uint2*>(base + kOffRanges);
     int* misc = reinterpret_cast<int*>(base + kOffMisc);
     int* status = misc;
     int* counter = misc + 4;
     uint32_t* dK = reinterpret_cast<uint32_t*>(misc + 12);
-
-    // scan levels for inputs up to max(n_views * T, 256 * sort blocks) = 2^16 items
-    ds::ScanScratch sc;
-    int64_t sizes[6] = {0};
-    sc.levels = ds::scan_levels(kMaxViewTris > 256 * kMaxSortBlocks ? kMaxViewTris : 256 * kMaxSortBlocks, sizes);
-    uint32_t* sp = reinterpret_cast<uint32_t*>(base + kOffScan);
-    for (int i = 0; i < sc.levels; ++i) {
-        sc.level_n[i] = sizes[i];
-        sc.level[i] = sp;
-        sp += sizes[i];
-        sc.level_out[i] = sp;
-        sp += sizes[i];
-    }
 
 #define NA_TRY(call)                                                                                         \
     do {                                                                                                    \
@@ -177,14 +159,13 @@ extern "C" DS_API ds_status ds_raster_forward_noalloc(const float* verts, const 
     } while (0)
 
     // ---- the forward pipeline of ds_raster_forward, on the scratch array.
-    // The array keeps the previous call's contents: the status word, the work
-    // counters and the tile ranges are cleared here.
-    const size_t nvt = (size_t)n_views * T;
+    // The array keeps the previous call's contents: the status word and the
+    // work counters are cleared here.
     NA_TRY(cudaMemsetAsync(misc, 0, 256, st));
     NA_TRY(ds::launch_activate(sd, st));
     ds::set_view_soups(vt, sd);
-    NA_TRY(ds::launch_setup(vt, recs, counts, tbox, zkeys, st));
-    NA_TRY(ds::scan_exclusive(counts, offs, (int64_t)nvt, dK, sc, st));
+    NA_TRY(ds::launch_setup(vt, tile_base, recs, tcount, tbox, zkeys, st));
+    NA_TRY(ds::launch_tile_offsets(tcount, tile_base, (uint32_t)kMaxPairs, tsums, ranges, tcursor, dK, counter, 2, st));
     uint32_t K = 0;   // the one data-dependent size, read back into host stack memory
     NA_TRY(cudaMemcpyAsync(&K, dK, sizeof(K), cudaMemcpyDeviceToHost, st));
     NA_TRY(cudaStreamSynchronize(st));
@@ -194,21 +175,16 @@ extern "C" DS_API ds_status ds_raster_forward_noalloc(const float* verts, const 
     int tile_bits = 0;
     while (tile_bits < 32 && (1ull << tile_bits) < (unsigned long long)tile_base) ++tile_bits;
     const int DB = tile_bits <= 16 ? 16 : 32 - tile_bits;
-    NA_TRY(ds::launch_emit(vt, recs, counts, offs, tbox, zkeys, DB, keys[0], vals[0], (uint32_t)kMaxPairs, status, st));
-    cudaError_t se = cudaSuccess;
-    const int res = ds::radix_sort_pairs(keys[0], vals[0], keys[1], vals[1], dK, K, tile_bits + DB, hist, hist_scan, sc,
-                                         st, &se);
-    NA_TRY(se);
-    NA_TRY(cudaMemsetAsync(ranges, 0, 8 * (size_t)tile_base, st));
-    NA_TRY(ds::launch_tile_ranges(keys[res], dK, K, DB, ranges, st));
+    NA_TRY(ds::launch_emit(vt, recs, tbox, zkeys, DB, tcursor, keys[0], vals[0], (uint32_t)kMaxPairs, status, st));
+    NA_TRY(ds::launch_tile_sort(ranges, tile_base, DB, keys[0], vals[0], keys[1], vals[1], st));
     ds::Bg b{};
     for (int i = 0; i < C - 1; ++i) b.c[i] = bg[i];
     const int grid = 0;
-    NA_TRY(ds::launch_raster_fwd(vt, sd, recs, keys[res], vals[res], ranges, DB, mode, b, counter, grid, st));
+    NA_TRY(ds::launch_raster_fwd(vt, sd, recs, keys[0], vals[0], ranges, DB, mode, b, counter, grid, st));
     bool want_front = false;
     for (int v = 0; v < n_views; ++v) want_front = want_front || out[v].n_front;
     if (want_front)
-        NA_TRY(ds::launch_raster_count(vt, sd, recs, keys[res], vals[res], ranges, DB, 0, nullptr, counter + 1, grid, st));
+        NA_TRY(ds::launch_raster_count(vt, sd, recs, keys[0], vals[0], ranges, DB, 0, nullptr, counter + 1, grid, st));
 #undef NA_TRY
     return DS_OK;
 }

@@ -178,7 +178,7 @@ __device__ __forceinline__ bool forward_walk(TileStage& sm, const SetupRec* __re
         const int n = (int)min((uint32_t)chunk, rg.y - c0);
         __syncthreads();
         if (tid < n)
-            stage_triangle<TW>(sm, tid, recs, vbase, keys[c0 + tid], vals[c0 + tid], DB, wi.tx * TW, wi.ty * TH);
+            stage_triangle<TW>(sm, tid, recs, vbase, DB > 0 ? keys[c0 + tid] : 0u, vals[c0 + tid], DB, wi.tx * TW, wi.ty * TH);
         __syncthreads();
         if (!warp_done) {
             for (int j = 0; j < n; ++j) {
@@ -441,7 +441,7 @@ __device__ __forceinline__ void score_walk(TileStage& sm, const SetupRec* __rest
             __syncthreads();
             if (!staged) {
                 if (tid < n)
-                    stage_triangle<TW>(sm, tid, recs, vbase, keys[c0 + tid], vals[c0 + tid], DB, wi.tx * TW,
+                    stage_triangle<TW>(sm, tid, recs, vbase, DB > 0 ? keys[c0 + tid] : 0u, vals[c0 + tid], DB, wi.tx * TW,
                                        wi.ty * TH);
                 __syncthreads();
             }
