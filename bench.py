@@ -135,7 +135,7 @@ class ClockSampler:
 
 
 # The sources the tile kernels (forward, backward, edge) are compiled from.
-TILE_KERNEL_SOURCES = ("ds_backward.cu", "ds_common.cuh", "ds_raster.cu", "ds_tile.cuh")
+TILE_KERNEL_SOURCES = ("ds_backward.cu", "ds_common.cuh", "ds_raster.cu", "ds_tile.cuh", "ds_walk.cuh")
 
 
 def _source_sha1() -> str:

@@ -315,7 +315,7 @@ int total_tiles(const ds::ViewTable& vt) {
 // tiles, in which a warp covers one row of 32 pixels and every per-pixel load
 // of a warp is one contiguous 128-byte line (the binning tiles of 8 x 32 cut
 // a warp's pixels into four 32-byte segments of four lines).
-constexpr int kEdgeTileW = 32;
+using ds::kEdgeTileW;
 
 void retile(const ds::ViewTable& vt, int tw, ds::ViewTable& out) {
     out = vt;

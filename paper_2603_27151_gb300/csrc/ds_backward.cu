@@ -518,7 +518,7 @@ __global__ void __launch_bounds__(kTilePix, DS_MINB_TRAIN)
             const int sg = s0 + q;
             reinterpret_cast<int4*>(V.gbuf)[sg * HW + pix] =
                 make_int4(bt[q], __float_as_int(bb1[q]), __float_as_int(bb2[q]), __float_as_int(bD[q]));
-            const float ell = color_loss_out(s, bt[q], bb1[q], bb2[q], bg, V.target + pix,
+            const float ell = color_loss_out<false>(s, bt[q], bb1[q], bb2[q], bg, V.target + pix,
                                              V.color + (size_t)sg * Co * HW + pix,
                                              const_cast<float*>(V.grad_color) + (size_t)sg * Co * HW + pix, HW,
                                              two_scale);
@@ -664,14 +664,14 @@ struct EdgeJob {
 // Ring capacity: up to 31 jobs left from earlier samples plus 4 per lane.
 constexpr int kJobsPerWarp = 5 * 32;
 
-template <int SG, int TW>
+template <int SG>
 __global__ void __launch_bounds__(kTilePix, DS_MINB_EDGE)
     k_edge_bwd(const __grid_constant__ ViewTable vt, const SoupDev s, const SetupRec* __restrict__ recs,
                const GeomRec* __restrict__ geom, double* __restrict__ acc_verts, int* __restrict__ counter) {
     __shared__ int s_item;
     __shared__ EdgeJob s_jobs[kTilePix / 32][kJobsPerWarp];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int TH = kTilePix / TW;
+    constexpr int TW = kEdgeTileW, TH = kTilePix / TW;
     const int lx = tid & (TW - 1), ly = tid / TW;
     const int Co = s.C - 1;
     EdgeJob* jobs = s_jobs[warp];
@@ -832,22 +832,25 @@ cudaError_t launch_raster_train(const ViewTable& vt, const SoupDev& s, const Set
                                 const uint32_t* vals, const uint2* ranges, int DB, uint32_t mode, const Bg& bg,
                                 float scale, float* loss, uint32_t flags, const GeomRec* geom, double* acc_tex,
                                 double* acc_verts, int* counter, int grid, cudaStream_t st) {
-    dispatch_tile(vt.tile_w, vt.S == 1 ? 1 : (vt.S == 2 ? 2 : 4), [&](auto P) {
-        constexpr int SG = decltype(P)::sg, TW = decltype(P)::tw;
-        k_raster_train<SG, TW><<<resident_grid(k_raster_train<SG, TW>, vt.n_items, grid), kTilePix, 0, st>>>(
+    const auto run = [&](auto kernel) {
+        kernel<<<resident_grid(kernel, vt.n_items, grid), kTilePix, 0, st>>>(
             vt, s, recs, keys, vals, ranges, DB, mode, bg, scale, loss, flags, geom, acc_tex, acc_verts, counter);
-    });
+    };
+    if (vt.tile_w == 8) run(k_raster_train<1, 8>);
+    else if (vt.tile_w == 32) run(k_raster_train<1, 32>);
+    else run(k_raster_train<1, 16>);
     note_launches(1);
     return cudaGetLastError();
 }
 
 cudaError_t launch_edge_bwd(const ViewTable& vt, const SoupDev& s, const SetupRec* recs, const GeomRec* geom,
                             double* acc_verts, int* counter, int grid, cudaStream_t st) {
-    dispatch_tile(vt.tile_w, vt.S == 1 ? 1 : (vt.S == 2 ? 2 : 4), [&](auto P) {
-        constexpr int SG = decltype(P)::sg, TW = decltype(P)::tw;
-        k_edge_bwd<SG, TW><<<resident_grid(k_edge_bwd<SG, TW>, vt.n_items, grid), kTilePix, 0, st>>>(
-            vt, s, recs, geom, acc_verts, counter);
-    });
+    const auto run = [&](auto kernel) {
+        kernel<<<resident_grid(kernel, vt.n_items, grid), kTilePix, 0, st>>>(vt, s, recs, geom, acc_verts, counter);
+    };
+    if (vt.S == 1) run(k_edge_bwd<1>);
+    else if (vt.S == 2) run(k_edge_bwd<2>);
+    else run(k_edge_bwd<4>);
     note_launches(1);
     return cudaGetLastError();
 }

@@ -36,6 +36,7 @@ void build_table(ViewTable& vt, const ds_tuning& tu, const ds_camera* cams, cons
 void note_launches(int n);
 long long launches_total();
 
+constexpr int kEdgeTileW = 32;      // tile width of the edge kernel (its own pixel partition)
 constexpr int kScanBlock = 4096;    // tiles per block of the tile scan (1024 threads x 4)
 
 // ---- activation (ds_activate.cu), set-up and binning (ds_bin.cu)
@@ -100,7 +101,7 @@ cudaError_t launch_raster_bwd(const ViewTable& vt, const SoupDev& s, const Setup
                               const uint32_t* keys, const uint32_t* vals, const uint2* ranges,
                               int DB, uint32_t flags, const GeomRec* geom, double* acc_tex,
                               double* acc_verts, int* counter, int grid, cudaStream_t st);
-// Fused training pass: forward + L2 loss + texture/score/interior gradients.
+// Fused training pass (S = 1): forward + L2 loss + texture/score/interior gradients.
 cudaError_t launch_raster_train(const ViewTable& vt, const SoupDev& s, const SetupRec* recs, const uint32_t* keys,
                                 const uint32_t* vals, const uint2* ranges, int DB, uint32_t mode, const Bg& bg,
                                 float scale, float* loss, uint32_t flags, const GeomRec* geom, double* acc_tex,

@@ -11,15 +11,20 @@ constexpr unsigned kFullMask = 0xffffffffu;
 
 // Resident CTAs per SM requested from the compiler for the tile kernels
 // (register budget 65536 / (256 x blocks)); set per kernel at build time.
-// The backward and the fused training pass run at five (48 registers):
-// their waits on gathers hide better with 40 warps than the spills cost;
-// the edge kernel and the forward of 4-sample groups are faster at four,
-// the forward of smaller groups (fewer registers per pixel) at five.
+// The backward and the fused training pass run at five (48 registers): their
+// waits on gathers hide better with 40 warps than the spills cost; the edge
+// kernel and the forward of 4-sample groups are faster at four.  The
+// warp-sized forward runs at five with one sample (149 us against 159 at four
+// and 174 at six on 200,000 triangles at 1080p) and at four with two (78
+// against 94 us at five, 80 at three on 8 small views).
 #ifndef DS_MINB_FWD
 #define DS_MINB_FWD 4
 #endif
-#ifndef DS_MINB_FWD_SMALL
-#define DS_MINB_FWD_SMALL 5
+#ifndef DS_MINB_WALK1
+#define DS_MINB_WALK1 5
+#endif
+#ifndef DS_MINB_WALK2
+#define DS_MINB_WALK2 4
 #endif
 #ifndef DS_MINB_BWD
 #define DS_MINB_BWD 5
@@ -251,8 +256,23 @@ __device__ __forceinline__ float winner_rho(const SetupRec* rec, int px, int py)
     return make_frag(E[0], E[1], E[2], r.k[0], r.k[1], r.k[2]).rho;
 }
 
-// Decode the C-1 colour channels of triangle t at (b1, b2) into out[c * HW].
-__device__ __forceinline__ void decode_color(const SoupDev& s, int t, float b1, float b2, float* out, size_t HW) {
+// for (c = 0; c < n; c += step) f(c), rolled or as the compiler likes.  The
+// CTA-tile kernels run fastest with the latter (their warps are in step, and
+// the loads of several samples overlap), the warp-sized forward with rolled
+// loops (small code).
+template <bool kRolled, class F>
+__device__ __forceinline__ void channel_loop(int n, int step, F&& f) {
+    if constexpr (kRolled) {
+#pragma unroll 1
+        for (int c = 0; c < n; c += step) f(c);
+    } else {
+        for (int c = 0; c < n; c += step) f(c);
+    }
+}
+
+// The C-1 interpolated colour channels of triangle t at (b1, b2): f(c, value).
+template <bool kRolled, class F>
+__device__ __forceinline__ void decode_channels(const SoupDev& s, int t, float b1, float b2, F&& f) {
     const Cell cl = find_cell(s.N, b1, b2);
     const int C = s.C;
     const float* base = s.act + (size_t)t * s.V * C;
@@ -260,7 +280,7 @@ __device__ __forceinline__ void decode_color(const SoupDev& s, int t, float b1, 
     const float* p1 = base + (size_t)cl.k1 * C;
     const float* p2 = base + (size_t)cl.k2 * C;
     if ((C & 3) == 0) {
-        for (int c4 = 0; c4 < C; c4 += 4) {
+        channel_loop<kRolled>(C, 4, [&](int c4) {
             const float4 a0 = __ldg(reinterpret_cast<const float4*>(p0 + c4));
             const float4 a1 = __ldg(reinterpret_cast<const float4*>(p1 + c4));
             const float4 a2 = __ldg(reinterpret_cast<const float4*>(p2 + c4));
@@ -268,56 +288,54 @@ __device__ __forceinline__ void decode_color(const SoupDev& s, int t, float b1, 
                                 interp(a0.z, a1.z, a2.z, cl.wa, cl.wb), interp(a0.w, a1.w, a2.w, cl.wa, cl.wb)};
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                if (c4 + k < C - 1) out[(c4 + k) * HW] = v[k];
-        }
+                if (c4 + k < C - 1) f(c4 + k, v[k]);
+        });
     } else {
-        for (int c = 0; c < C - 1; ++c)
-            out[c * HW] = interp(__ldg(p0 + c), __ldg(p1 + c), __ldg(p2 + c), cl.wa, cl.wb);
+        channel_loop<kRolled>(C - 1, 1, [&](int c) {
+            f(c, interp(__ldg(p0 + c), __ldg(p1 + c), __ldg(p2 + c), cl.wa, cl.wb));
+        });
     }
 }
 
-// Colour of the selected fragment (or the background), written to col[c*HW],
-// with the per-pixel L2 loss against tgt[c*HW] and its upstream gradient
-// gc[c*HW] = 2 scale (colour - target); returns l = sum_c (colour - target)^2.
-// Same arithmetic, in the same order, as the forward's decode followed by
-// ds_loss_l2.
+// Background channels: f(c, bg.c[c]).
+template <bool kRolled, class F>
+__device__ __forceinline__ void background_channels(const Bg& bg, int Co, F&& f) {
+    if constexpr (kRolled) {
+#pragma unroll 1
+        for (int c = 0; c < Co; ++c) f(c, bg.c[c]);
+    } else {
+#pragma unroll
+        for (int c = 0; c < DS_MAX_CHANNELS; ++c)   // constant indices into the parameter struct
+            if (c < Co) f(c, bg.c[c]);
+    }
+}
+
+// Colour of the selected fragment (or the background), written to col[c*HW].
+template <bool kRolled>
+__device__ __forceinline__ void color_out(const SoupDev& s, int t, float b1, float b2, const Bg& bg,
+                                          float* __restrict__ col, size_t HW) {
+    const auto emit = [&](int c, float v) { col[c * HW] = v; };
+    if (t < 0) background_channels<kRolled>(bg, s.C - 1, emit);
+    else decode_channels<kRolled>(s, t, b1, b2, emit);
+}
+
+// The same with the per-pixel L2 loss against tgt[c*HW] and its upstream
+// gradient gc[c*HW] = 2 scale (colour - target); returns l = sum_c (colour -
+// target)^2.  Same arithmetic, in the same order, as the forward's decode
+// followed by ds_loss_l2.
+template <bool kRolled>
 __device__ __forceinline__ float color_loss_out(const SoupDev& s, int t, float b1, float b2, const Bg& bg,
                                                 const float* __restrict__ tgt, float* __restrict__ col,
                                                 float* __restrict__ gc, size_t HW, float two_scale) {
-    const int Co = s.C - 1;
     float ell = 0.f;
-    auto emit = [&](int c, float v) {
+    const auto emit = [&](int c, float v) {
         col[c * HW] = v;
         const float d = __fsub_rn(v, __ldg(tgt + c * HW));
         ell = __fmaf_rn(d, d, ell);
         gc[c * HW] = __fmul_rn(two_scale, d);
     };
-    if (t < 0) {
-#pragma unroll
-        for (int c = 0; c < DS_MAX_CHANNELS; ++c)   // constant indices into the parameter struct
-            if (c < Co) emit(c, bg.c[c]);
-        return ell;
-    }
-    const Cell cl = find_cell(s.N, b1, b2);
-    const int C = s.C;
-    const float* base = s.act + (size_t)t * s.V * C;
-    const float* p0 = base + (size_t)cl.k0 * C;
-    const float* p1 = base + (size_t)cl.k1 * C;
-    const float* p2 = base + (size_t)cl.k2 * C;
-    if ((C & 3) == 0) {
-        for (int c4 = 0; c4 < C; c4 += 4) {
-            const float4 a0 = __ldg(reinterpret_cast<const float4*>(p0 + c4));
-            const float4 a1 = __ldg(reinterpret_cast<const float4*>(p1 + c4));
-            const float4 a2 = __ldg(reinterpret_cast<const float4*>(p2 + c4));
-            const float v[4] = {interp(a0.x, a1.x, a2.x, cl.wa, cl.wb), interp(a0.y, a1.y, a2.y, cl.wa, cl.wb),
-                                interp(a0.z, a1.z, a2.z, cl.wa, cl.wb), interp(a0.w, a1.w, a2.w, cl.wa, cl.wb)};
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (c4 + k < Co) emit(c4 + k, v[k]);
-        }
-    } else {
-        for (int c = 0; c < Co; ++c) emit(c, interp(__ldg(p0 + c), __ldg(p1 + c), __ldg(p2 + c), cl.wa, cl.wb));
-    }
+    if (t < 0) background_channels<kRolled>(bg, s.C - 1, emit);
+    else decode_channels<kRolled>(s, t, b1, b2, emit);
     return ell;
 }
 
