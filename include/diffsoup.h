@@ -477,7 +477,7 @@ DS_API ds_status ds_get_shade_path(ds_ctx* ctx, int32_t* path);
  *   grad_color = scale * d(sum_p ell_p)/d color  (non-local: the window).
  *  Arguments and layouts as ds_loss_l2 (C counts the opacity channel: C-1
  *  colour channels).  grad_colors, score_ws and loss may be NULL.  FP32; one
- *  fused pass per 32 x 16 tile.  Allocates nothing on the device. */
+ *  fused pass.  Allocates nothing on the device. */
 DS_API ds_status ds_loss_l1_ssim(int32_t n_views, int32_t S, int32_t C, const int32_t* hw,
                                  const float* const* colors, const float* const* targets,
                                  float* const* grad_colors, float* const* score_ws, float lambda, float scale,
