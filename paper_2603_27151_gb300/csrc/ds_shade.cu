@@ -434,13 +434,25 @@ __global__ void __launch_bounds__(kThreads, 2) k_shade_bwd(const __grid_constant
     }
 }
 
-// grad_params[k] (+)= sum over CTAs of partial[c][k], in FP64, CTA order.
-__global__ void __launch_bounds__(kThreads) k_shade_finish(const float* __restrict__ partial, int n_cta,
-                                                            float* __restrict__ out, int overwrite) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= kParams) return;
+// grad_params[k] (+)= sum over CTAs of partial[c][k] in FP64, in a fixed order:
+// warp w of the block sums the CTAs w, w + 16, ... for 32 parameters, and the
+// 16 sums are added in order.  A thread per parameter over all 304 partials was
+// one long chain of loads (49 us; 10 now).
+constexpr int kFinWarps = 16;
+__global__ void __launch_bounds__(32 * kFinWarps) k_shade_finish(const float* __restrict__ partial, int n_cta,
+                                                                 float* __restrict__ out, int overwrite) {
+    __shared__ double s_sum[kFinWarps][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k = blockIdx.x * 32 + lane;
     double a = 0.0;
-    for (int c = 0; c < n_cta; ++c) a += (double)partial[(size_t)c * kParams + k];
+    if (k < kParams) {
+#pragma unroll 4
+        for (int c = warp; c < n_cta; c += kFinWarps) a += (double)partial[(size_t)c * kParams + k];
+    }
+    s_sum[warp][lane] = a;
+    __syncthreads();
+    if (warp > 0 || k >= kParams) return;
+#pragma unroll
+    for (int w = 1; w < kFinWarps; ++w) a += s_sum[w][lane];
     out[k] = overwrite ? (float)a : (float)((double)out[k] + a);
 }
 
@@ -869,8 +881,7 @@ cudaError_t launch_shade_bwd(const ShadeView* views, int n, int S, const float* 
         note_launches(1);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if (grad_params) {
-            k_shade_finish<<<(kParams + kThreads - 1) / kThreads, kThreads, 0, st>>>(partial, g, grad_params,
-                                                                                   overwrite ? 1 : 0);
+            k_shade_finish<<<(kParams + 31) / 32, 32 * kFinWarps, 0, st>>>(partial, g, grad_params, overwrite ? 1 : 0);
             note_launches(1);
         }
     } else if (grad_params && overwrite) {
