@@ -132,13 +132,7 @@ struct SoupDev {
 // power-of-two factors.
 __device__ __forceinline__ float pow2i(int k) { return __int_as_float((k + 127) << 23); }
 
-__device__ __forceinline__ float pinned_exp(float x) {
-    if (x != x) return x;
-    if (x >= 0x1.62e430p+6f) return __int_as_float(0x7f800000);
-    if (x < -0x1.9fe368p+6f) return 0.0f;
-    const float kf = rintf(__fmul_rn(x, 0x1.715476p+0f));
-    float r = __fmaf_rn(-kf, 0x1.62e400p-1f, x);
-    r = __fmaf_rn(-kf, 0x1.7f7d1cp-20f, r);
+__device__ __forceinline__ float exp_poly(float r) {
     float p = 0x1.a01a02p-13f;
     p = __fmaf_rn(p, r, 0x1.6c16c2p-10f);
     p = __fmaf_rn(p, r, 0x1.111112p-7f);
@@ -146,16 +140,35 @@ __device__ __forceinline__ float pinned_exp(float x) {
     p = __fmaf_rn(p, r, 0x1.555556p-3f);
     p = __fmaf_rn(p, r, 0.5f);
     p = __fmaf_rn(p, r, 1.0f);
-    p = __fmaf_rn(p, r, 1.0f);
-    const int k = (int)kf;
-    const int k1 = k / 2, k2 = k - k1;
-    return __fmul_rn(__fmul_rn(p, pow2i(k1)), pow2i(k2));
+    return __fmaf_rn(p, r, 1.0f);
 }
 
-// Sigmoid of Sec. 3.3, applied per feature vertex before rasterisation.
-__device__ __forceinline__ float pinned_sigmoid(float th) {
-    return __fdiv_rn(1.0f, __fadd_rn(1.0f, pinned_exp(-th)));
+__device__ __forceinline__ float pinned_exp(float x) {
+    const float t = __fmul_rn(x, 0x1.715476p+0f);
+    if (fabsf(x) < 80.0f) {
+        // The same value without the conversions of rintf and int (both on the
+        // quarter-rate pipe of the special functions): adding and taking off
+        // 1.5 * 2^23 rounds t to an integer (to even), whose two's complement
+        // then sits in the low bits; e^r 2^k stays normal here, so that one
+        // scaling is exact like the two of the general form.
+        const float m = __fadd_rn(t, 0x1.8p+23f);
+        const float kf = __fsub_rn(m, 0x1.8p+23f);
+        const float r = __fmaf_rn(-kf, 0x1.7f7d1cp-20f, __fmaf_rn(-kf, 0x1.62e400p-1f, x));
+        return __fmul_rn(exp_poly(r), __int_as_float((__float_as_int(m) + 127) << 23));
+    }
+    if (x != x) return x;
+    if (x >= 0x1.62e430p+6f) return __int_as_float(0x7f800000);
+    if (x < -0x1.9fe368p+6f) return 0.0f;
+    const float kf = rintf(t);
+    const float r = __fmaf_rn(-kf, 0x1.7f7d1cp-20f, __fmaf_rn(-kf, 0x1.62e400p-1f, x));
+    const int k = (int)kf;
+    const int k1 = k / 2, k2 = k - k1;
+    return __fmul_rn(__fmul_rn(exp_poly(r), pow2i(k1)), pow2i(k2));
 }
+
+// Sigmoid of Sec. 3.3, applied per feature vertex before rasterisation.  The
+// correctly rounded reciprocal is the IEEE division 1 / (1 + e^-x).
+__device__ __forceinline__ float pinned_sigmoid(float th) { return __frcp_rn(__fadd_rn(1.0f, pinned_exp(-th))); }
 
 // Philox4x32-10 block (Salmon et al., SC'11).
 __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1) {
@@ -181,6 +194,17 @@ struct Cell {
 
 __device__ __forceinline__ int texel_index(int N, int i, int j) {
     return ((j * (2 * N + 3 - j)) >> 1) + i;   // j (N + 1) - j (j - 1) / 2 + i
+}
+
+// (i, j) of vertex v of the N-subdivided grid (rows of constant j).
+__device__ __forceinline__ void texel_ij(int N, int v, int& i, int& j) {
+    const float b = (float)(2 * N + 3);
+    int jj = (int)floorf(0.5f * (b - sqrtf(b * b - 8.0f * (float)v)));
+    jj = jj < 0 ? 0 : (jj > N ? N : jj);
+    while (jj > 0 && texel_index(N, 0, jj) > v) --jj;
+    while (jj < N && texel_index(N, 0, jj + 1) <= v) ++jj;
+    j = jj;
+    i = v - texel_index(N, 0, jj);
 }
 
 // Rounding towards minus infinity into int32 saturates (NaN gives 0), so the

@@ -35,17 +35,6 @@ namespace {
 
 __host__ __device__ constexpr int level_V(int R) { return ((1 << R) + 1) * ((1 << R) + 2) / 2; }
 
-// (i, j) of vertex v of the N-subdivided grid (rows of constant j).
-__device__ __forceinline__ void texel_ij(int N, int v, int& i, int& j) {
-    const float b = (float)(2 * N + 3);
-    int jj = (int)floorf(0.5f * (b - sqrtf(b * b - 8.0f * (float)v)));
-    jj = jj < 0 ? 0 : (jj > N ? N : jj);
-    while (jj > 0 && texel_index(N, 0, jj) > v) --jj;
-    while (jj < N && texel_index(N, 0, jj + 1) <= v) ++jj;
-    j = jj;
-    i = v - texel_index(N, 0, jj);
-}
-
 // Value of channel c of the level-R grid g ([V_R][C]) at vertex (i, j) of
 // the grid with N = 2^k subdivisions.
 __device__ __forceinline__ float level_value(const float* __restrict__ g, int R, int C, int c, int i, int j, int N) {
@@ -95,11 +84,6 @@ __host__ __device__ inline int stage_floats(int r_min, int r_max, int C) {
     for (int R = r_min; R <= r_max; ++R) n += level_V(R) * C;
     return n;
 }
-
-// Sigmoid of Sec. 3.3 with the reciprocal of (1 + e^-x) taken by the
-// correctly rounded reciprocal: the same value as pinned_sigmoid's IEEE
-// division 1 / (1 + e^-x) (both round 1/y to nearest; y >= 1).
-__device__ __forceinline__ float sigmoid_rcp(float th) { return __frcp_rn(__fadd_rn(1.0f, pinned_exp(-th))); }
 
 // Tap of one coarse level at one finest vertex, shared by every triangle:
 // corner texel indices k0 | k1 << 10 | k2 << 20 (| 1 << 30 when the vertex
@@ -173,7 +157,10 @@ __global__ void __launch_bounds__(256, 5) k_compose(const float* __restrict__ le
     float* const stage0 = smem + tap_floats;                               // stage b at stage0 + b * sf
     size_t fine_off = 0;                                                   // the finest level in `levels`
     for (int R = r_min; R < r_max; ++R) fine_off += (size_t)T * level_V(R) * C;
+    // item = (vertex, channel group); a thread's items are 256 apart
     const int per = C / 4;
+    const int v0 = threadIdx.x / per, g0 = threadIdx.x - v0 * per;
+    const int dv = blockDim.x / per, dg = blockDim.x - dv * per;
     int t = blockIdx.x;
     if (t < T) stage_coarse(stage0, levels, t, T, r_min, r_max, C);
     cp_async_commit();
@@ -192,8 +179,12 @@ __global__ void __launch_bounds__(256, 5) k_compose(const float* __restrict__ le
         __syncthreads();      // everyone's (and the taps)
         const float* zs = stage0 + buf * sf;
         const float* fine = levels + fine_off + (size_t)t * Vf * C;
-        for (int it = threadIdx.x; it < Vf * per; it += blockDim.x) {
-            const int v = it / per, c = (it - v * per) * 4;
+        for (int v = v0, g = g0; v < Vf; v += dv, g += dg) {
+            if (g >= per) {
+                g -= per;
+                if (++v >= Vf) break;
+            }
+            const int c = 4 * g;
             const float4 y = __ldcs(reinterpret_cast<const float4*>(fine + (size_t)v * C + c));
             float4 z = tap_value(zs, taps[v], C, c);
             int so = level_V(r_min) * C;
@@ -203,7 +194,7 @@ __global__ void __launch_bounds__(256, 5) k_compose(const float* __restrict__ le
             }
             z = add4(z, y);
             if (kAct) {
-                z = make_float4(sigmoid_rcp(z.x), sigmoid_rcp(z.y), sigmoid_rcp(z.z), sigmoid_rcp(z.w));
+                z = make_float4(pinned_sigmoid(z.x), pinned_sigmoid(z.y), pinned_sigmoid(z.z), pinned_sigmoid(z.w));
                 if (c + 4 == C && act_a) act_a[(size_t)t * Vf + v] = z.w;
             }
             __stcs(reinterpret_cast<float4*>(out + ((size_t)t * Vf + v) * C + c), z);
@@ -288,6 +279,32 @@ __device__ __forceinline__ float restrict_value(const float* G, int N, int k, in
     return fmaf(0.5f, half, acc);
 }
 
+// The same for channels c .. c + 3 of vertex u (each in restrict_value's order).
+__device__ __forceinline__ float4 restrict_value4(const float* G, int N, int u, int c, int C) {
+    const int Nfine = 2 * N;
+    int a, b;
+    texel_ij(N, u, a, b);
+    const int x = 2 * a, y = 2 * b;
+    const auto at = [&](int xi, int yi) {
+        return *reinterpret_cast<const float4*>(G + (size_t)texel_index(Nfine, xi, yi) * C + c);
+    };
+    const float4 acc = at(x, y);
+    float4 half = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int dx[6] = {1, -1, 0, 0, 1, -1}, dy[6] = {0, 0, 1, -1, -1, 1};
+#pragma unroll
+    for (int e = 0; e < 6; ++e) {
+        const int xi = x + dx[e], yi = y + dy[e];
+        if (xi < 0 || yi < 0 || xi + yi > Nfine) continue;
+        const float4 g = at(xi, yi);
+        half.x += g.x;
+        half.y += g.y;
+        half.z += g.z;
+        half.w += g.w;
+    }
+    return make_float4(fmaf(0.5f, half.x, acc.x), fmaf(0.5f, half.y, acc.y), fmaf(0.5f, half.z, acc.z),
+                       fmaf(0.5f, half.w, acc.w));
+}
+
 // Adjoint of the composition for one triangle per CTA.  fine: FP64 gradient
 // of the composed logits [T][V_f][C]; out: the level gradients (same layout
 // as the levels), written or accumulated.
@@ -354,7 +371,7 @@ __global__ void __launch_bounds__(256) k_restrict(const double* __restrict__ fin
 template <bool kAdam>
 __global__ void __launch_bounds__(256) k_restrict_staged(const double* __restrict__ fine, int T, int r_min, int r_max,
                                                          int C, float* __restrict__ out, AdamTex adam) {
-    extern __shared__ float sm[];   // the levels' gradients of this triangle, finest first
+    extern __shared__ __align__(16) float sm[];   // the levels' gradients of this triangle, finest first
     const int t = blockIdx.x;
     size_t off[6];
     int soff[6];
@@ -371,20 +388,20 @@ __global__ void __launch_bounds__(256) k_restrict_staged(const double* __restric
         }
     }
     {
-        const int n = level_V(r_max) * C;
-        const double* src = fine + (size_t)t * n;
-        float* G = sm + soff[r_max - r_min];
-        for (int k0 = threadIdx.x; k0 < n; k0 += 8 * blockDim.x) {
-            double g[8];
+        const int n2 = level_V(r_max) * C / 2;
+        const double2* src = reinterpret_cast<const double2*>(fine) + (size_t)t * n2;
+        float2* G = reinterpret_cast<float2*>(sm + soff[r_max - r_min]);
+        for (int k0 = threadIdx.x; k0 < n2; k0 += 4 * blockDim.x) {
+            double2 g[4];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
+            for (int u = 0; u < 4; ++u) {
                 const int k = k0 + u * blockDim.x;
-                g[u] = k < n ? __ldcs(src + k) : 0.0;
+                g[u] = k < n2 ? __ldcs(src + k) : make_double2(0.0, 0.0);
             }
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
+            for (int u = 0; u < 4; ++u) {
                 const int k = k0 + u * blockDim.x;
-                if (k < n) G[k] = (float)g[u];
+                if (k < n2) G[k] = make_float2((float)g[u].x, (float)g[u].y);
             }
         }
     }
@@ -392,8 +409,11 @@ __global__ void __launch_bounds__(256) k_restrict_staged(const double* __restric
     for (int R = r_max - 1; R >= r_min; --R) {
         const float* Gf = sm + soff[R + 1 - r_min];
         float* G = sm + soff[R - r_min];
-        const int n = level_V(R) * C;
-        for (int k = threadIdx.x; k < n; k += blockDim.x) G[k] = restrict_value(Gf, 1 << R, k, C);
+        const int n4 = level_V(R) * C / 4, per = C / 4;
+        for (int q = threadIdx.x; q < n4; q += blockDim.x) {
+            const int u = q / per;
+            reinterpret_cast<float4*>(G)[q] = restrict_value4(Gf, 1 << R, u, 4 * (q - u * per), C);
+        }
         __syncthreads();
     }
     // each level's block, four values per access (the block starts on a
