@@ -17,6 +17,7 @@
 //    children of a split edge (midpoint in FP32), each child's grid sampled
 //    from the parent's grid at the child's vertices mapped into the parent.
 #include <algorithm>
+#include <type_traits>
 #include <numeric>
 #include <vector>
 
@@ -118,32 +119,95 @@ __device__ __forceinline__ void child_corners(int op, int P[3][3]) {
         for (int q = 0; q < 3; ++q) P[i][q] = Q[i][q];
 }
 
-__global__ void __launch_bounds__(256) k_rebuild_level(const float* __restrict__ gin, int N, int C,
+// Where a texel of a child comes from: one parent texel (k, all ones above
+// bit 10), or the decode's interpolation of the three in k's ten-bit fields.
+struct RebuildTap {
+    unsigned k;
+    float wa, wb;
+};
+constexpr unsigned kOneTexel = 0xfffffc00u;
+constexpr int kRebuildItems = 2;   // items in flight per thread
+
+// One level.  The source of a child's texel depends on its code and vertex
+// only: every CTA tabulates the six splits first (shared memory), then the
+// items, V texels of C / 4 channel groups per triangle (scalar channels when
+// C or the alignment does not allow 16 bytes), stream through it with
+// consecutive lanes on consecutive addresses.  Bound by the latency of the
+// gathers and by HBM: level 5 of 20,000 triangles (718 MB, 107 us at the copy
+// rate) 375 -> 131 us against one thread per texel with an index search and
+// scalar channels.  Two items in flight per thread at five CTAs per SM; one:
+// 141 us, three: 268 us, four at two CTAs: 255 us.
+template <bool kVec>
+__global__ void __launch_bounds__(256, 5) k_rebuild_level(const float* __restrict__ gin, int N, int C,
                                                        const int* __restrict__ plan, int n_out,
                                                        float* __restrict__ gout) {
+    extern __shared__ RebuildTap taps[];   // [6][V]
     const int V = (N + 1) * (N + 2) / 2;
-    const long long n = (long long)n_out * V;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n;
-         q += (long long)gridDim.x * blockDim.x) {
-        const int k = (int)(q / V), v = (int)(q - (long long)k * V);
-        int j = 0;
-        while (j < N && texel_index(N, 0, j + 1) <= v) ++j;
-        const int i = v - texel_index(N, 0, j);
-        const int code = __ldg(plan + k), parent = code >> 3, op = code & 7;
+    for (int q = threadIdx.x; q < 6 * V; q += blockDim.x) {
+        const int op = q / V + 1, v = q - (op - 1) * V;
+        int i, j;
+        texel_ij(N, v, i, j);
         int P[3][3];
         child_corners(op, P);
         const int X = (N - i - j) * P[0][1] + i * P[1][1] + j * P[2][1];
         const int Y = (N - i - j) * P[0][2] + i * P[1][2] + j * P[2][2];
-        const float* g = gin + (size_t)parent * V * C;
-        float* d = gout + (size_t)q * C;
         if ((X & 1) == 0 && (Y & 1) == 0) {
-            const float* s = g + (size_t)texel_index(N, X >> 1, Y >> 1) * C;
-            for (int c = 0; c < C; ++c) d[c] = __ldg(s + c);
+            taps[q] = RebuildTap{kOneTexel | (unsigned)texel_index(N, X >> 1, Y >> 1), 0.f, 0.f};
         } else {
             const Cell cl = find_cell(N, __fdiv_rn((float)X, (float)(2 * N)), __fdiv_rn((float)Y, (float)(2 * N)));
-            for (int c = 0; c < C; ++c)
-                d[c] = interp(__ldg(g + (size_t)cl.k0 * C + c), __ldg(g + (size_t)cl.k1 * C + c),
-                              __ldg(g + (size_t)cl.k2 * C + c), cl.wa, cl.wb);
+            taps[q] = RebuildTap{(unsigned)(cl.k0 | (cl.k1 << 10) | (cl.k2 << 20)), cl.wa, cl.wb};
+        }
+    }
+    __syncthreads();
+    // items: channel group c of texel r of output triangle k; a thread keeps
+    // its channel group (the grid's threads are a multiple of `per`)
+    const int per = kVec ? C / 4 : C;
+    const unsigned id = blockIdx.x * blockDim.x + threadIdx.x, threads = gridDim.x * blockDim.x;
+    const unsigned c = id % per, step = threads / per;   // in texels
+    const int dk = (int)(step / V), dr = (int)(step - (unsigned)dk * V);
+    int k = (int)(id / per / V), r = (int)(id / per - (unsigned)k * V);
+    using Item = std::conditional_t<kVec, float4, float>;
+    const Item* in = reinterpret_cast<const Item*>(gin) + c;
+    Item* out = reinterpret_cast<Item*>(gout) + c;
+    while (k < n_out) {
+        Item a[kRebuildItems], b[kRebuildItems], d[kRebuildItems];
+        RebuildTap tp[kRebuildItems];
+        size_t dst[kRebuildItems];
+        int n = 0;
+#pragma unroll
+        for (int u = 0; u < kRebuildItems; ++u) {
+            if (k < n_out) {
+                n = u + 1;
+                const int code = __ldg(plan + k), op = code & 7;
+                tp[u] = op > 0 ? taps[(op - 1) * V + r] : RebuildTap{kOneTexel | (unsigned)r, 0.f, 0.f};
+                const Item* g = in + (size_t)(code >> 3) * (unsigned)(V * per);
+                a[u] = __ldg(g + (tp[u].k & 1023u) * per);
+                if (tp[u].k < kOneTexel) {
+                    b[u] = __ldg(g + ((tp[u].k >> 10) & 1023u) * per);
+                    d[u] = __ldg(g + ((tp[u].k >> 20) & 1023u) * per);
+                }
+                dst[u] = ((size_t)k * V + r) * per;
+                k += dk;
+                r += dr;
+                if (r >= V) {
+                    r -= V;
+                    ++k;
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kRebuildItems; ++u) {
+            if (u >= n) break;
+            if (tp[u].k < kOneTexel) {
+                if constexpr (kVec)
+                    a[u] = make_float4(interp(a[u].x, b[u].x, d[u].x, tp[u].wa, tp[u].wb),
+                                       interp(a[u].y, b[u].y, d[u].y, tp[u].wa, tp[u].wb),
+                                       interp(a[u].z, b[u].z, d[u].z, tp[u].wa, tp[u].wb),
+                                       interp(a[u].w, b[u].w, d[u].w, tp[u].wa, tp[u].wb));
+                else
+                    a[u] = interp(a[u], b[u], d[u], tp[u].wa, tp[u].wb);
+            }
+            __stcs(out + dst[u], a[u]);
         }
     }
 }
@@ -171,12 +235,6 @@ __global__ void __launch_bounds__(256) k_rebuild_verts(const float* __restrict__
         d[3 + q] = c == 0 ? m[q] : __ldg(s + 3 * b + q);
         d[6 + q] = __ldg(s + 3 * o + q);
     }
-}
-
-int flat_grid(long long n) {
-    long long g = (n + 255) / 256;
-    if (g > 152 * 16) g = 152 * 16;
-    return g < 1 ? 1 : (int)g;
 }
 
 }  // namespace
@@ -226,8 +284,23 @@ cudaError_t launch_rebuild(const float* verts, const float* tex, int T, const in
     size_t off_in = 0, off_out = 0;
     for (int l = 0; l < n_levels; ++l) {
         const int N = grid_ns[l], V = (N + 1) * (N + 2) / 2;
-        k_rebuild_level<<<flat_grid((long long)n_out * V), 256, 0, st>>>(tex + off_in, N, C, plan_dev, n_out,
-                                                                          tex_out + off_out);
+        const float* in = tex + off_in;
+        float* out = tex_out + off_out;
+        const bool vec = C % 4 == 0 && (((uintptr_t)in | (uintptr_t)out) & 15) == 0;
+        const size_t smem = sizeof(RebuildTap) * 6 * (size_t)V;
+        const auto run = [&](auto kernel) {
+            cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+            const int per = vec ? C / 4 : C;
+            const long long items = (long long)n_out * V * per;
+            // at least eight items per thread; a multiple of `per` CTAs
+            long long grid = std::min<long long>((items + 2047) / 2048, persistent_grid(1 << 30, 5));
+            grid = (grid + per - 1) / per * per;
+            kernel<<<(unsigned)grid, 256, smem, st>>>(in, N, C, plan_dev, n_out, out);
+            return cudaGetLastError();
+        };
+        const cudaError_t e = vec ? run(k_rebuild_level<true>) : run(k_rebuild_level<false>);
+        if (e != cudaSuccess) return e;
         note_launches(1);
         off_in += (size_t)T * V * C;
         off_out += (size_t)n_out * V * C;
