@@ -21,7 +21,7 @@
 //
 // Tiles of 64 x 16 pixels on their own blur 2.6 rows per row horizontally and
 // 1.9 vertically (549 M against 310 M warp instructions on four 1080p images
-// of three channels).  There 735 -> 505 us; issue active 55%, FMA pipe 31% (a
+// of three channels).  There 735 -> 527 us; issue active 55%, FMA pipe 31% (a
 // packed FMA takes two of its cycles), shared-memory wavefronts 50% of their
 // peak, one CTA of 16 warps per SM.
 //
@@ -75,7 +75,7 @@ struct SsimSmem {
     float Gb[kStep][kGX];        // G3
     float2 ga[kKeep][kHX];       // horizontal pass of (G1, G2): 10 rows kept, 16 new
     float gb[kKeep][kHX];        // of G3
-    float P[kMaxRows][kTX];      // per pixel, summed over channels: lambda |x - y| - (1 - lambda) ssim
+    float P[kMaxRows][kTX];      // ssim, summed over channels
 };
 static_assert(sizeof(SsimSmem) <= 227 * 1024, "shared memory of one CTA");
 static_assert(kMX == 128 && kThreads == 4 * kMX && kThreads == 32 * kStep, "one task per thread");
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_loss_l1_ssim(const __grid_const
                     g2 = dvar;
                     g3 = dcov;
                     if ((unsigned)ry < (unsigned)rows && (unsigned)(vq - kR) < (unsigned)kTX)
-                        sm.P[ry][vq - kR] -= (1.f - t.lambda) * ssim;
+                        sm.P[ry][vq - kR] += ssim;
                 }
                 sm.Ga[r][vs] = make_float2(g1, g2);
                 sm.Gb[r][vq] = g3;
@@ -285,9 +285,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_loss_l1_ssim(const __grid_const
         }
         if (nc < t.Co) store_regs(buf ^ 1);
         __syncthreads();
-        // ---- vertical pass onto the image: gradient and the L1 term (the
-        // pixels' colours once more, from L2)
-        if (st > 0 && vq < kTX) {
+        // ---- vertical pass onto the image: the gradient (the pixels' colours
+        // once more, from L2)
+        if (V.grad_color && st > 0 && vq < kTX) {
             const int ry0 = kStep * st - 4 * kR + vr;
             const bool col_in = x0 + vq < V.W;
             const long long pix = (long long)(y0 + ry0) * V.W + (x0 + vq);
@@ -321,13 +321,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_loss_l1_ssim(const __grid_const
                 if ((unsigned)ry >= (unsigned)rows || !col_in) continue;
                 const float x = X[o], y = Y[o];
                 const float d = x - y;
-                sm.P[ry][vq] += t.lambda * fabsf(d);
-                if (V.grad_color) {
-                    const float dsum = A[o].x + 2.f * x * A[o].y + y * B[o];
-                    const float sg = d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f);
-                    const float gval = (t.lambda * sg - (1.f - t.lambda) * dsum) / (float)t.Co;
-                    gout[(size_t)o * V.W] = t.scale * gval;
-                }
+                const float dsum = A[o].x + 2.f * x * A[o].y + y * B[o];
+                const float sg = d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f);
+                const float gval = (t.lambda * sg - (1.f - t.lambda) * dsum) / (float)t.Co;
+                gout[(size_t)o * V.W] = t.scale * gval;
             }
         }
         // no barrier here: the next horizontal pass touches nothing that the
@@ -339,12 +336,31 @@ __global__ void __launch_bounds__(kThreads, 1) k_loss_l1_ssim(const __grid_const
     __syncthreads();   // P complete
     // per-pixel loss, score weight, total
     float acc = 0.f;
-    for (int k = tid; k < rows * kTX; k += kThreads) {
-        const int r = k / kTX, q = k - r * kTX, gx = x0 + q;
-        if (gx >= V.W) continue;
-        const float ell = (1.f - t.lambda) + sm.P[r][q] / (float)t.Co;
-        if (V.score_w) V.score_w[(size_t)s * HW + (size_t)(y0 + r) * V.W + gx] = t.scale * ell;
-        acc += ell;
+    if (vq < kTX && x0 + vq < V.W) {
+        // the L1 sum from the colours again (L2): folding it into P channel by
+        // channel saves this read (505 us) but rounds the sum another way.
+        // Eight pixels per thread at a time for the loads' latency (one at a
+        // time: 565 us)
+        constexpr int kBatch = 8;
+        const float* xs = V.color + (size_t)s * t.Co * HW + (size_t)y0 * V.W + x0 + vq;
+        const float* ys = V.target + (size_t)y0 * V.W + x0 + vq;
+        for (int r0 = tid / kMX; r0 < rows; r0 += 4 * kBatch) {
+            float l1[kBatch] = {};
+            for (int ch = 0; ch < t.Co; ++ch)
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) {
+                    const size_t o = ch * HW + (size_t)min(r0 + 4 * u, rows - 1) * V.W;
+                    l1[u] += fabsf(__ldg(xs + o) - __ldg(ys + o));
+                }
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+                const int r = r0 + 4 * u;
+                if (r >= rows) break;
+                const float ell = t.lambda * l1[u] / (float)t.Co + (1.f - t.lambda) * (1.f - sm.P[r][vq] / (float)t.Co);
+                if (V.score_w) V.score_w[(size_t)s * HW + (size_t)(y0 + r) * V.W + x0 + vq] = t.scale * ell;
+                acc += ell;
+            }
+        }
     }
     if (loss) {
 #pragma unroll
