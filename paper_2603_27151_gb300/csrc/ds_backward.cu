@@ -563,37 +563,68 @@ __device__ __forceinline__ void add_world(const DevCam& cam, f3 gc, float* out) 
     out[2] += gw.z;
 }
 
-// Contribution of side X of a pixel pair (X -> Y along unit axis e = (ex, ey))
-// whose winner triangle is t: silhouette or mask-induced (implicit) boundary.
-// phi = 1/2 sum_c (g_X + g_Y)(C_X - C_Y).  Returns false if X is not in front.
-// Every array index is a compile-time constant (no local memory).
-__device__ __forceinline__ bool edge_side(const DevCam& cam, const SetupRec* vrec, const GeomRec* g, int t, int xX,
-                                          int yX, int xY, int yY, int tY, float phi, float (&out)[9]) {
-    const SetupRec r = load_rec(vrec + t);
-    long long E[3];
-    const float ex = (float)(xY - xX), ey = (float)(yY - yX);
-    if (cover_exact(r, xY, yY, E)) {
-        const float rho = make_frag(E[0], E[1], E[2], r.k[0], r.k[1], r.k[2]).rho;
-        if (tY >= 0 && !in_front(rho, t, winner_rho(vrec + tY, xY, yY), tY)) return false;   // occluded at Y
-        // implicit boundary: the material point under the pair's midpoint
-        // moves with the surface; weight 1 per pair axis
-        float dx, dy, beta[3], inv;
-        ray_bary(g, cam, 0.5f * (float)(xX + xY + 1), 0.5f * (float)(yX + yY + 1), dx, dy, beta, inv);
-        const f3 e1 = ld3(g->e1), e2 = ld3(g->e2), v0 = ld3(g->v0);
-        const f3 P = mk3(v0.x + beta[1] * e1.x + beta[2] * e2.x, v0.y + beta[1] * e1.y + beta[2] * e2.y,
-                         v0.z + beta[1] * e1.z + beta[2] * e2.z);
-        const float iz = 1.0f / P.z;
-        // J^T e with J rows (fx/z, 0, -fx x/z^2), (0, fy/z, -fy y/z^2)
-        const f3 je = mk3(ex * cam.fx * iz, ey * cam.fy * iz, -(ex * cam.fx * P.x + ey * cam.fy * P.y) * iz * iz);
+// A side of a pixel pair (X -> Y along a unit axis) whose winner X has triangle
+// t; tY: winner at Y (-1: background); phi = 1/2 sum_c (g_X + g_Y)(C_X - C_Y)
+// for side X.  xyd: x | y << 13 | direction << 26, the direction Y - X =
+// (1, 0) / (-1, 0) / (0, 1) / (0, -1) as 0..3.
+struct __align__(16) EdgeJob {
+    unsigned xyd;
+    int t, tY;
+    float phi;
+};
+static_assert(DS_MAX_RESOLUTION <= 1 << 13, "pixel coordinates of an edge job");
+__device__ __forceinline__ EdgeJob make_job(int x, int y, int dir, int t, int tY, float phi) {
+    return EdgeJob{(unsigned)x | ((unsigned)y << 13) | ((unsigned)dir << 26), t, tY, phi};
+}
+__device__ __forceinline__ void job_pixels(const EdgeJob& jb, int& xX, int& yX, int& ex, int& ey) {
+    const int dir = (int)(jb.xyd >> 26);
+    xX = (int)(jb.xyd & 8191u);
+    yX = (int)((jb.xyd >> 13) & 8191u);
+    ex = (dir == 0) - (dir == 1);
+    ey = (dir == 2) - (dir == 3);
+}
+
+// What side X is: 0 occluded at Y, 1 a mask-induced (implicit) boundary -- its
+// triangle covers Y in front of Y's winner -- 2 a silhouette.
+__device__ __forceinline__ int edge_class(const SetupRec* vrec, const EdgeJob& jb) {
+    int xX, yX, ex, ey;
+    job_pixels(jb, xX, yX, ex, ey);
+    const SetupRec r = load_rec(vrec + jb.t);
+    float e[3];
+    if (!cover_near(r, xX + ex, yX + ey, e)) return 2;
+    const float rho = edge_frag(e[0], e[1], e[2], r.k[0], r.k[1], r.k[2]).rho;
+    if (jb.tY >= 0 && !in_front(rho, jb.t, winner_rho(vrec + jb.tY, xX + ex, yX + ey), jb.tY)) return 0;
+    return 1;
+}
+
+// Implicit boundary: the material point under the pair's midpoint moves with
+// the surface; weight 1 per pair axis.
+__device__ __forceinline__ void edge_implicit(const DevCam& cam, const GeomRec* g, const EdgeJob& jb, float (&out)[9]) {
+    int xX, yX, ix, iy;
+    job_pixels(jb, xX, yX, ix, iy);
+    const float ex = (float)ix, ey = (float)iy;
+    float dx, dy, beta[3], inv;
+    ray_bary(g, cam, 0.5f * (float)(2 * xX + ix + 1), 0.5f * (float)(2 * yX + iy + 1), dx, dy, beta, inv);
+    const f3 e1 = ld3(g->e1), e2 = ld3(g->e2), v0 = ld3(g->v0);
+    const f3 P = mk3(v0.x + beta[1] * e1.x + beta[2] * e2.x, v0.y + beta[1] * e1.y + beta[2] * e2.y,
+                     v0.z + beta[1] * e1.z + beta[2] * e2.z);
+    const float iz = 1.0f / P.z;
+    // J^T e with J rows (fx/z, 0, -fx x/z^2), (0, fy/z, -fy y/z^2)
+    const f3 je = mk3(ex * cam.fx * iz, ey * cam.fy * iz, -(ex * cam.fx * P.x + ey * cam.fy * P.y) * iz * iz);
 #pragma unroll
-        for (int m = 0; m < 3; ++m) {
-            const float f = phi * beta[m];
-            add_world(cam, mk3(f * je.x, f * je.y, f * je.z), out + 3 * m);
-        }
-        return true;
+    for (int m = 0; m < 3; ++m) {
+        const float f = jb.phi * beta[m];
+        add_world(cam, mk3(f * je.x, f * je.y, f * je.z), out + 3 * m);
     }
-    // silhouette: the first edge the segment X -> Y crosses; coordinates
-    // relative to X's pixel centre
+}
+
+// Silhouette: the first edge that the segment X -> Y crosses; coordinates
+// relative to X's pixel centre.  Every array index is a compile-time constant
+// (no local memory).
+__device__ __forceinline__ void edge_silhouette(const DevCam& cam, const GeomRec* g, const EdgeJob& jb, float (&out)[9]) {
+    int xX, yX, ix, iy;
+    job_pixels(jb, xX, yX, ix, iy);
+    const float ex = (float)ix, ey = (float)iy;
     const float cxX = (float)xX + 0.5f, cyX = (float)yX + 0.5f;
     float sx[3], sy[3];
 #pragma unroll
@@ -623,12 +654,12 @@ __device__ __forceinline__ bool edge_side(const DevCam& cam, const SetupRec* vre
             by = sy[b];
         }
     }
-    if (best < 0) return true;
+    if (best < 0) return;
     const float fX = bfX * sg, fY = bfY * sg;
     const float den = (fX - fY) * (fX - fY);
     const float ux = bx - ax, uy = by - ay;
     const float omega = (ex != 0.f ? uy * uy : ux * ux) / (ux * ux + uy * uy);
-    const float k = omega * phi / den;
+    const float k = omega * jb.phi / den;
     // d f(x)/d a = (b_y - x_y, -(b_x - x_x)); d f(x)/d b = (-(a_y - x_y), a_x - x_x)
     const float gax = k * (fX * (by - ey) - fY * by), gay = k * (fX * (-(bx - ex)) - fY * (-bx));
     const float gbx = k * (fX * (-(ay - ey)) - fY * (-ay)), gby = k * (fX * (ax - ex) - fY * ax);
@@ -642,39 +673,49 @@ __device__ __forceinline__ bool edge_side(const DevCam& cam, const SetupRec* vre
         const float k0 = __ldg(&g->jy[m][0]), k1 = __ldg(&g->jy[m][1]);
         add_world(cam, mk3(gx * j0, gy * k0, gx * j1 + gy * k1), out + 3 * m);
     }
-    return true;
 }
 
 // One CTA per (view, tile, sample group); every pixel owns its pairs with
 // the right and the lower neighbour.  A pair with different winners yields up
 // to two side jobs (one per side with a triangle).  Each warp queues its jobs
-// in a ring in shared memory (prefix over lanes) and evaluates them 32 at a
-// time whenever 32 are waiting, across the samples of the work item, so that
-// every lane works on a boundary instead of idling; only the last batch of a
-// work item can be partial.  Consecutive jobs mostly share a triangle, and
-// runs of equal triangles are summed before the atomics.
-struct EdgeJob {
-    int xy;      // X: x | (y << 16)
-    int t;       // triangle of side X
-    int tY;      // winner at Y (-1: background)
-    float phi;   // 1/2 sum_c (g_X + g_Y)(C_X - C_Y) for side X
-    int dir;     // Y = X + (1, 0) / (-1, 0) / (0, 1) / (0, -1): 0..3
-};
+// in a ring in shared memory (prefix over lanes), across the samples of the
+// work item, and works on them 64 at a time (two per lane; fewer at the item's
+// end): it finds out what each side is, then evaluates the implicit and the
+// silhouette ones separately, 32 per round, and puts the results back in the
+// jobs' order.  The two kinds share no code, so that a mixed batch ran both
+// paths with half the lanes idle; 64 jobs fill the rounds of both.
+// Consecutive jobs mostly share a triangle: runs of equal triangles within 32
+// jobs are summed before the atomics.
+//
+// Bound by instruction issue and the latency of the records that a job reads
+// (4 CTAs of 64 registers per SM; 3 or 5 are slower).  Together with the 32-bit
+// cover test 2774 -> 2456 us for 100k triangles, four views of 1080p and four
+// of 960 x 540, S = 4; 302 -> 281 us for 20k triangles, four views of
+// 1024 x 768, S = 1.  Rings of their own for the two kinds, summed as they
+// come, are faster still (2274 us) but regroup the FP32 run sums, and a last
+// bit of a vertex gradient can change a later step's visibility.
 
-// Ring capacity: up to 31 jobs left from earlier samples plus 4 per lane.
-constexpr int kJobsPerWarp = 5 * 32;
+// Up to 63 jobs left from earlier samples plus 4 per lane.
+constexpr int kJobsPerWarp = 6 * 32;
+
+struct EdgeScratch {
+    EdgeJob jobs[kJobsPerWarp];
+    float out[9][64];             // the jobs' vertex gradients
+    unsigned char list[2][64];    // the implicit jobs, the silhouette jobs
+};
 
 template <int SG>
 __global__ void __launch_bounds__(kTilePix, DS_MINB_EDGE)
     k_edge_bwd(const __grid_constant__ ViewTable vt, const SoupDev s, const SetupRec* __restrict__ recs,
                const GeomRec* __restrict__ geom, double* __restrict__ acc_verts, int* __restrict__ counter) {
     __shared__ int s_item;
-    __shared__ EdgeJob s_jobs[kTilePix / 32][kJobsPerWarp];
+    __shared__ EdgeScratch s_scratch[kTilePix / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned lt = (1u << lane) - 1u;
     constexpr int TW = kEdgeTileW, TH = kTilePix / TW;
     const int lx = tid & (TW - 1), ly = tid / TW;
     const int Co = s.C - 1;
-    EdgeJob* jobs = s_jobs[warp];
+    EdgeScratch& sc = s_scratch[warp];
     for (;;) {
         if (tid == 0) s_item = atomicAdd(counter, 1);
         __syncthreads();
@@ -738,11 +779,11 @@ __global__ void __launch_bounds__(kTilePix, DS_MINB_EDGE)
                 const float phi = phid[dir];
                 if (phi == 0.f) continue;
                 if (tp >= 0) {
-                    sl[dir] = EdgeJob{px | (py << 16), tp, tq, phi, dir == 0 ? 0 : 2};
+                    sl[dir] = make_job(px, py, dir == 0 ? 0 : 2, tp, tq, phi);
                     vl[dir] = true;
                 }
                 if (tq >= 0) {
-                    sl[2 + dir] = EdgeJob{qx | (qy << 16), tq, tp, -phi, dir == 0 ? 1 : 3};
+                    sl[2 + dir] = make_job(qx, qy, dir == 0 ? 1 : 3, tq, tp, -phi);
                     vl[2 + dir] = true;
                 }
             }
@@ -758,26 +799,54 @@ __global__ void __launch_bounds__(kTilePix, DS_MINB_EDGE)
             pre -= nmine;
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                if (vl[k]) jobs[(head + count + pre++) % kJobsPerWarp] = sl[k];
+                if (vl[k]) sc.jobs[(head + count + pre++) % kJobsPerWarp] = sl[k];
             count += total;
             __syncwarp();
-            // ---- evaluate 32 at a time while a full batch waits (and the
-            // remainder after the last sample)
-            while (count >= 32 || (q == SG - 1 && count > 0)) {
-                const int n = min(count, 32);
-                float acc[9];
+            // ---- 64 at a time (and the remainder after the last sample)
+#pragma unroll 1
+            while (count >= 64 || (q == SG - 1 && count > 0)) {
+                const int n = min(count, 64);
+                int nk[2] = {0, 0};   // implicit, silhouette jobs
+                unsigned on = 0;      // this lane's jobs that count (bit u: job 32 u + lane)
+#pragma unroll 1
+                for (int u = 0; u < 2; ++u) {
+                    const int j = 32 * u + lane;
+                    int cls = 0;
+                    if (j < n) cls = edge_class(vrec, sc.jobs[(head + j) % kJobsPerWarp]);
+                    on |= cls > 0 ? 1u << u : 0u;
 #pragma unroll
-                for (int k = 0; k < 9; ++k) acc[k] = 0.f;
-                bool act = false;
-                int t = -1;
-                if (lane < n) {
-                    const EdgeJob jb = jobs[(head + lane) % kJobsPerWarp];
-                    const int xX = jb.xy & 0xffff, yX = jb.xy >> 16;
-                    const int xY = xX + (jb.dir == 0) - (jb.dir == 1), yY = yX + (jb.dir == 2) - (jb.dir == 3);
-                    t = jb.t;
-                    act = edge_side(view_cam(vt, wi.v), vrec, vgeom + t, t, xX, yX, xY, yY, jb.tY, jb.phi, acc);
+                    for (int k = 0; k < 2; ++k) {
+                        const unsigned m = __ballot_sync(kFullMask, cls == k + 1);
+                        if (cls == k + 1) sc.list[k][nk[k] + __popc(m & lt)] = (unsigned char)j;
+                        nk[k] += __popc(m);
+                    }
                 }
-                scatter_verts_run(acc_verts, act, t, acc);
+                __syncwarp();
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+#pragma unroll 1
+                    for (int i = lane; i < nk[k]; i += 32) {
+                        const int j = sc.list[k][i];
+                        const EdgeJob jb = sc.jobs[(head + j) % kJobsPerWarp];
+                        float acc[9];
+#pragma unroll
+                        for (int c = 0; c < 9; ++c) acc[c] = 0.f;
+                        if (k == 0) edge_implicit(view_cam(vt, wi.v), vgeom + jb.t, jb, acc);
+                        else edge_silhouette(view_cam(vt, wi.v), vgeom + jb.t, jb, acc);
+#pragma unroll
+                        for (int c = 0; c < 9; ++c) sc.out[c][j] = acc[c];
+                    }
+                }
+                __syncwarp();
+#pragma unroll 1
+                for (int u = 0; u < 2; ++u) {
+                    const int j = 32 * u + lane;
+                    const bool act = (on >> u) & 1u;
+                    float acc[9];
+#pragma unroll
+                    for (int c = 0; c < 9; ++c) acc[c] = act ? sc.out[c][j] : 0.f;
+                    scatter_verts_run(acc_verts, act, act ? sc.jobs[(head + j) % kJobsPerWarp].t : -1, acc);
+                }
                 head = (head + n) % kJobsPerWarp;
                 count -= n;
                 __syncwarp();

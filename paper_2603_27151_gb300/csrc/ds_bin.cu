@@ -146,6 +146,10 @@ __global__ void __launch_bounds__(256) k_setup(const __grid_constant__ ViewTable
                 r.B[i] = B;
                 r.C[i] = Cc;
             }
+            const int amax = max(max(max(abs(r.A[0]), abs(r.A[1])), abs(r.A[2])), max(max(abs(r.B[0]), abs(r.B[1])), abs(r.B[2])));
+            const int cx = (X[0] >> kCellBits) + 1, cy = (Y[0] >> kCellBits) + 1;
+            if (amax <= kSmallEdge && (unsigned)cx < 256u && (unsigned)cy < 256u)
+                r.bias |= kSmallTri | ((uint32_t)cx << 4) | ((uint32_t)cy << 12);
             const float fa = __ll2float_rn(area > 0 ? area : -area);
 #pragma unroll
             for (int i = 0; i < 3; ++i) r.k[i] = __fdiv_rn(__fdiv_rn(1.0f, w[i]), fa);

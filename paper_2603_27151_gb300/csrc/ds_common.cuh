@@ -93,8 +93,15 @@ struct __align__(16) SetupRec {
     int32_t B[3];
     long long C[3];
     float k[3];
-    uint32_t bias;   // bit i set: edge i is not owned (bias 1 folded into C_i)
+    uint32_t bias;   // bit i set: edge i is not owned (bias 1 folded into C_i); bits 3..19: kSmallTri
 };
+// Bit 3: no edge is longer than 63 pixels in x or y; bits 4..11 and 12..19 are
+// then 1 + the cell of 64 x 64 pixels of vertex 0.  Within that cell and the
+// eight around it, which hold every pixel that the triangle covers, the edge
+// values fit int32: |2 area| + 256 * 2 * 128 * max(|A|, |B|) < 2^31.
+constexpr uint32_t kSmallTri = 8u;
+constexpr int kSmallEdge = 63 * 256, kCellBits = 14;
+static_assert(2LL * kSmallEdge * kSmallEdge + 256LL * 2 * 128 * kSmallEdge + 1 < 1LL << 31, "int32 edge values");
 static_assert(sizeof(SetupRec) == 64, "SetupRec must be 64 bytes");
 
 // Continuous (unsnapped) geometry of one (view, triangle) for the vertex
@@ -246,9 +253,6 @@ __device__ __forceinline__ Frag edge_frag(float e0, float e1, float e2, float k0
     f.rho = __fadd_rn(__fadd_rn(q0, f.q1), f.q2);
     return f;
 }
-__device__ __forceinline__ Frag make_frag(long long e0, long long e1, long long e2, float k0, float k1, float k2) {
-    return edge_frag(__ll2float_rn(e0), __ll2float_rn(e1), __ll2float_rn(e2), k0, k1, k2);
-}
 
 // (rho, t) is in front of (rho2, t2): larger inverse depth, then lower index.
 __device__ __forceinline__ bool in_front(float rho, int t, float rho2, int t2) {
@@ -266,6 +270,29 @@ __device__ __forceinline__ bool cover_exact(const SetupRec& r, int px, int py, l
         cov = cov && (eb >= 0);
         E[i] = eb + ((r.bias >> i) & 1u);
     }
+    return cov;
+}
+
+// The same with the values rounded once, in int32 where the record and the
+// pixel allow it.
+__device__ __forceinline__ bool cover_near(const SetupRec& r, int px, int py, float e[3]) {
+    const unsigned dx = (unsigned)((px >> 6) + 2) - ((r.bias >> 4) & 255u);
+    const unsigned dy = (unsigned)((py >> 6) + 2) - ((r.bias >> 12) & 255u);
+    if ((r.bias & kSmallTri) && dx <= 2u && dy <= 2u) {
+        const uint32_t X = 256u * px + 128u, Y = 256u * py + 128u;
+        int low = 0;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const int eb = (int)((uint32_t)r.A[i] * X + ((uint32_t)r.B[i] * Y + (uint32_t)r.C[i]));
+            low |= eb;
+            e[i] = __int2float_rn(eb + (int)((r.bias >> i) & 1u));
+        }
+        return low >= 0;
+    }
+    long long E[3];
+    const bool cov = cover_exact(r, px, py, E);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) e[i] = __ll2float_rn(E[i]);
     return cov;
 }
 

@@ -251,9 +251,9 @@ __device__ __forceinline__ bool forward_walk(TileStage& sm, const SetupRec* __re
 // key, recomputed bit for bit).  +inf if the record does not cover the pixel.
 __device__ __forceinline__ float winner_rho(const SetupRec* rec, int px, int py) {
     const SetupRec r = load_rec(rec);
-    long long E[3];
-    if (!cover_exact(r, px, py, E)) return __int_as_float(0x7f800000);
-    return make_frag(E[0], E[1], E[2], r.k[0], r.k[1], r.k[2]).rho;
+    float e[3];
+    if (!cover_near(r, px, py, e)) return __int_as_float(0x7f800000);
+    return edge_frag(e[0], e[1], e[2], r.k[0], r.k[1], r.k[2]).rho;
 }
 
 // for (c = 0; c < n; c += step) f(c), rolled or as the compiler likes.  The

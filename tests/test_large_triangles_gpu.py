@@ -71,3 +71,33 @@ def test_backward_matches_oracle(ctx, S):
     gt, _ = gpu_backward(ctx, sid, sc, S, g, col, gc, sw, 3, verts, tex)   # texture and score terms
     gt_ref, _ = O.backward(sc.verts, sc.tex, sc.grid_n, sc.cams, S, ref, gc, sw, flags=3)
     assert not grad_mismatch(gt, gt_ref).any()
+
+
+@pytest.mark.parametrize("S", [1, 2, 4])
+def test_edge_gradients_around_the_int32_limit(ctx, S):
+    """Edge terms of triangles below and above the size up to which boundary
+    tests run in int32 (edges of 63 pixels), with |2 area| around 2^30 and
+    edges around 2^21 (in 1/256 pixels); two views."""
+    rng = np.random.default_rng(11)
+    tri = []
+    for k, (w, h) in enumerate([(128, 127), (128, 128), (130, 128), (64, 256), (24, 8180), (24, 8200), (30, 40)]):
+        x, y, z = 5.0 + 11.0 * k, -30.0 * (h > 1000) + 9.0 * k, 1.0 + 0.04 * k
+        tri.append([(x, y, z), (x + w, y + 3, z + 0.1), (x + 4, y + h, z + 0.2)])
+    tri += [[a, c, b] for a, b, c in tri]
+    t = np.array(tri)
+    t[7:, :, 2] += 0.03
+    cams = [I.Camera(w, h, 64.0, 64.0, cx, 0.0, np.eye(3, dtype=np.float32), np.zeros(3, np.float32))
+            for w, h, cx in ((150, 140, 0.0), (97, 61, 12.25))]
+    verts = np.stack([t[..., 0] * t[..., 2] / 64.0, t[..., 1] * t[..., 2] / 64.0, t[..., 2]], -1).astype(np.float32)
+    s = np.round(t[..., :2] * 256).astype(np.int64)
+    area = np.abs((s[:, 1, 0] - s[:, 0, 0]) * (s[:, 2, 1] - s[:, 0, 1]) - (s[:, 2, 0] - s[:, 0, 0]) * (s[:, 1, 1] - s[:, 0, 1]))
+    assert (area < 2 ** 30).any() and (area >= 2 ** 30).any()
+    tex = I.logits(len(verts), 8, 4, rng)
+    sc = I.Scene(verts, tex, 8, cams, I.mask_seeds(3, 2), 1, np.zeros(3, np.float32))
+    sid, got, (g, col, vd, td) = gpu_forward(ctx, sc, S=S)
+    ref = O.forward(sc.verts, sc.tex, sc.grid_n, sc.cams, sc.seeds, S=S, bg=sc.bg)
+    assert_forward_equal(got, ref)
+    gc, sw = upstream(ref, S)
+    _, gv = gpu_backward(ctx, sid, sc, S, g, col, gc, sw, 8, vd, td)   # edge terms
+    _, gv_ref = O.backward(sc.verts, sc.tex, sc.grid_n, sc.cams, S, ref, gc, sw, flags=8)
+    assert not grad_mismatch(gv, gv_ref).any()
