@@ -14,9 +14,10 @@
 //  - the SH half of the first layer does not depend on the mask sample: it is
 //    evaluated once per pixel and reused for all S samples;
 //  - the parameters sit in shared memory and are read as float4 broadcasts,
-//    each load shared by two samples of the same pixel;
+//    each load shared by two samples of a pixel (forward) or by two pixels
+//    (backward);
 //  - the backward stages each round's activations and deltas in shared memory
-//    and reduces the weight gradients as 4x4 outer-product blocks per thread
+//    and reduces the weight gradients as 4x8 outer-product blocks per thread
 //    over the CTA's pixels, into one FP32 partial per CTA; a finish kernel
 //    sums the partials in FP64 in a fixed order (deterministic gradients).
 #include <string>
@@ -184,41 +185,83 @@ __global__ void __launch_bounds__(kThreads) k_shade_fwd(const __grid_constant__ 
 // ---------------------------------------------------------------------------
 // Backward.
 //
-// Staging per round (one sample of the CTA's 256 pixels), row-major [p][20]:
-// X (input: features, SH), H1, H2, D1 = dL/dz1, D2 = dL/dz2, D3 = dL/dz3
-// (padded to 4).  Reduction: threads 0..251 = 7 pixel groups x 36 blocks;
-// block b < 16 owns gW1[4(b/4)..][4(b%4)..] (+ gb1 if b%4 == 0), 16 <= b < 32
-// the same of gW2, 32 <= b < 36 gW3[0..2][4(b-32)..] (+ gb3 if b == 32).
-constexpr int kGroups = 7, kBlocks = 36;
+// A CTA of 128 threads takes 256 pixels, two per thread, one sample a round.
+// Staging per round, row-major [p][20]: X (input: features, SH), H1, H2,
+// D1 = dL/dz1, D2 = dL/dz2, and D3 = dL/dz3 (padded to 4).  Reduction: 7 pixel
+// groups x 16 blocks of 4 x 8 weights; block b < 8 owns gW1[4(b/2)..][8(b%2)..]
+// (+ gb1 if b is even), b >= 8 the same of gW2, and each block a column of gW3
+// (+ gb3 if b = 0).
+//
+// Bound by the shared-memory pipe, then by the FMA pipe.  With one pixel per
+// thread and 4 x 4 blocks a weight load fed four multiply-adds and a reducer's
+// two loads sixteen: 840 shared wavefronts per 32 pixel-samples, 74% of the
+// pipe's peak, FMA pipe at 40%.  Here a weight load feeds four outputs of two
+// pixels, a reducer's three loads 32 multiply-adds, and two multiply-adds are
+// one packed instruction: in the layers the weights of neighbouring outputs
+// are pairs (stored transposed for the forward) and the activation is in both
+// halves; in a reducer the products (d0, d1) x (a0, a1) and (d1, d0) x (a0, a1)
+// give all four.  Every sum keeps its order: the layers that of the forward
+// kernel, the weight gradients the rows 7 apart of the CTA's blocks.
+// Four 1080p views and one of 1023 x 577, S = 2: 1958 -> 1555 us (shared 60% of
+// its peak, FMA pipe's issue 30% at two cycles per packed instruction, issue
+// 47%; 8 warps per SM, as 224 registers and 108 KB per CTA allow).  16 pixel
+// groups x 8 blocks of 8 x 8 were faster (1440) but sum in another order.
+constexpr int kPix = kThreads;           // pixels of a block
+constexpr int kBwdThreads = kPix / 2;
+constexpr int kGroups = 7, kBlocks = 16;
 constexpr int kRow = 20;   // 16 values + 4 pad: conflict-free float4 stores of the rows
 
-// A warp of reducers reads one row of D1 and of D2 (and of X and of H1) at
-// once: the 64-byte pads put those arrays on complementary shared-memory banks.
+// A warp of reducers reads two rows of D1 and D2 (of X and H1) at once: the
+// 64-byte pads put those arrays on complementary shared-memory banks.
 struct BwdSmem {
     float sp[kParamsPad];
-    float X[kThreads][kRow];
+    float W1T[kIn][kHid], W2T[kHid][kHid], W3T[kHid][4];   // [input][output]
+    float X[kPix][kRow];
     float pad0[16];
-    float H1[kThreads][kRow], H2[kThreads][kRow], D1[kThreads][kRow];
+    float H1[kPix][kRow], H2[kPix][kRow], D1[kPix][kRow];
     float pad1[16];
-    float D2[kThreads][kRow];
-    float D3[kThreads][4];
+    float D2[kPix][kRow];
+    float D3[kPix][4];
 };
-static_assert(sizeof(float) * kGroups * kParams <= sizeof(float) * (2 * kThreads * kRow + 16), "reduction buffer");
+static_assert(sizeof(float) * kGroups * kParams <= sizeof(float) * (2 * kPix * kRow + 16), "reduction buffer");
+static_assert(2 * (sizeof(BwdSmem) + 1024) <= 228 * 1024, "two CTAs per SM");
 
 // The sample-independent part of the first layer (16 values per pixel) kept
-// in the 4 pad columns of the thread's X, H1, H2 and D1 rows (the reducers
+// in the 4 pad columns of the pixel's X, H1, H2 and D1 rows (the reducers
 // read columns 0..15 only).
-__device__ __forceinline__ float* upad(BwdSmem& sm, int tid, int q) {
-    return q == 0 ? &sm.X[tid][16] : q == 1 ? &sm.H1[tid][16] : q == 2 ? &sm.H2[tid][16] : &sm.D1[tid][16];
+__device__ __forceinline__ float4* upad(BwdSmem& sm, int row, int q) {
+    return reinterpret_cast<float4*>(q == 0 ? &sm.X[row][16] : q == 1 ? &sm.H1[row][16] : q == 2 ? &sm.H2[row][16] : &sm.D1[row][16]);
 }
 
 __device__ __forceinline__ void store4(float* dst, const float* v) {
     *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
 }
 
-__global__ void __launch_bounds__(kThreads, 2) k_shade_bwd(const __grid_constant__ ShadeTable t,
-                                                            const float* __restrict__ params,
-                                                            float* __restrict__ partial) {
+// acc[i] += (w[2 i], w[2 i + 1]) x for N pairs of weights in shared memory and
+// the two pixels' x.
+template <int N>
+__device__ __forceinline__ void fma_pairs(const float* w, float x0, float x1, float2 (&a0)[N], float2 (&a1)[N]) {
+    const float2 xx0 = make_float2(x0, x0), xx1 = make_float2(x1, x1);
+#pragma unroll
+    for (int i = 0; i < N; i += 2) {
+        const float4 v = *reinterpret_cast<const float4*>(w + 2 * i);
+        a0[i] = __ffma2_rn(make_float2(v.x, v.y), xx0, a0[i]);
+        a1[i] = __ffma2_rn(make_float2(v.x, v.y), xx1, a1[i]);
+        a0[i + 1] = __ffma2_rn(make_float2(v.z, v.w), xx0, a0[i + 1]);
+        a1[i + 1] = __ffma2_rn(make_float2(v.z, v.w), xx1, a1[i + 1]);
+    }
+}
+__device__ __forceinline__ float elem(const float2* a, int i) { return i & 1 ? a[i >> 1].y : a[i >> 1].x; }
+template <int N>
+__device__ __forceinline__ void store_pairs(float* dst, const float2 (&a)[N]) {
+#pragma unroll
+    for (int i = 0; i < N; i += 2)
+        reinterpret_cast<float4*>(dst)[i / 2] = make_float4(a[i].x, a[i].y, a[i + 1].x, a[i + 1].y);
+}
+
+__global__ void __launch_bounds__(kBwdThreads, 2) k_shade_bwd(const __grid_constant__ ShadeTable t,
+                                                               const float* __restrict__ params,
+                                                               float* __restrict__ partial) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     BwdSmem& sm = *reinterpret_cast<BwdSmem*>(smem_raw);
     const float* sp = sm.sp;
@@ -226,207 +269,248 @@ __global__ void __launch_bounds__(kThreads, 2) k_shade_bwd(const __grid_constant
 
     const int tid = threadIdx.x;
     const int grp = tid / kBlocks, blk = tid % kBlocks;
-    const bool reducer = tid < kGroups * kBlocks;
-    const int layer = blk >> 4;                       // 0: W1, 1: W2, 2: W3
-    const int ib = layer < 2 ? (blk >> 2) & 3 : 0;    // row block
-    const int jb = layer < 2 ? blk & 3 : blk - 32;    // column block
-    const int nrow = layer < 2 ? 4 : kOut;
-    const bool bias_owner = (jb == 0);
-    const float* Dsrc = layer == 0 ? &sm.D1[0][0] : layer == 1 ? &sm.D2[0][0] : &sm.D3[0][0];
-    const float* Asrc = layer == 0 ? &sm.X[0][0] : layer == 1 ? &sm.H1[0][0] : &sm.H2[0][0];
-    const int dstride = layer < 2 ? kRow : 4;
-    float acc[4][4], accb[4];
+    const bool reducer = grp < kGroups;
+    const int layer = blk >> 3;                             // 0: W1, 1: W2
+    const int ib = (blk >> 1) & 3, jb = blk & 1;            // row block, column block
+    const float* Dsrc = (layer == 0 ? &sm.D1[0][0] : &sm.D2[0][0]) + 4 * ib;
+    const float* Asrc = (layer == 0 ? &sm.X[0][0] : &sm.H1[0][0]) + 8 * jb;
+    float2 accP[2][4], accQ[2][4], accb[2];   // (d0 a0, d1 a1); (d1 a0, d0 a1); (d0, d1)
+    float2 acc3 = make_float2(0.f, 0.f), accb3 = make_float2(0.f, 0.f);   // gW3[0, 1][blk], gb3[0, 1]
+    float acc3z = 0.f, accb3z = 0.f;                                      // the third output's
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        accb[i] = 0.f;
+    for (int i = 0; i < 2; ++i) {
+        accb[i] = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+        for (int j = 0; j < 4; ++j) accP[i][j] = accQ[i][j] = make_float2(0.f, 0.f);
     }
     __syncthreads();
+    for (int k = tid; k < kHid * kIn; k += kBwdThreads) {
+        sm.W1T[k % kIn][k / kIn] = sp[oW1 + k];
+        sm.W2T[k % kHid][k / kHid] = sp[oW2 + k];
+    }
+    for (int k = tid; k < 4 * kHid; k += kBwdThreads) sm.W3T[k >> 2][k & 3] = (k & 3) < kOut ? sp[oW3 + (k & 3) * kHid + (k >> 2)] : 0.f;
+    __syncthreads();
 
+    // A round's features and gradients are loaded before the reduction of the
+    // round before it, where registers are free.
+    float f[2][8], g[2][kOut];
+    const auto load = [&](int b, int s) {
+        const ShadeView& V = t.v[find_view(t, b)];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int p = (b - V.blk0) * kPix + e * kBwdThreads + tid;
+            const bool valid = p < V.HW;
+#pragma unroll
+            for (int c = 0; c < kFeat; ++c) f[e][c] = valid ? __ldg(V.feat + ((size_t)s * kFeat + c) * V.HW + p) : 0.f;
+#pragma unroll
+            for (int c = 0; c < kOut; ++c) g[e][c] = valid ? __ldcs(V.grad_rgb + ((size_t)s * kOut + c) * V.HW + p) : 0.f;
+        }
+    };
+    load(blockIdx.x, 0);
+#pragma unroll 1
     for (int b = blockIdx.x; b < t.n_blocks; b += gridDim.x) {
         const ShadeView& V = t.v[find_view(t, b)];
-        const int p = (b - V.blk0) * kThreads + tid;
-        const bool valid = p < V.HW;
+        int p[2];
+        bool valid[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            p[e] = (b - V.blk0) * kPix + e * kBwdThreads + tid;
+            valid[e] = p[e] < V.HW;
+        }
         {
             // the SH columns 8..15 of the input row are the same for every
             // sample (column 7, the constant band, is stored with the features)
-            float sh[kSH + 3] = {};
-            float u[kHid];
-            if (valid) {
-                sh_of_pixel(V, p % V.W, p / V.W, sh);
-                first_layer_sh(sp, sh, u);
+            float sh[2][kSH] = {};
+            float2 u[2][kHid / 2];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) store4(upad(sm, tid, q), u + 4 * q);
+            for (int e = 0; e < 2; ++e) {
+                if (valid[e]) sh_of_pixel(V, p[e] % V.W, p[e] / V.W, sh[e]);
+                store4(&sm.X[e * kBwdThreads + tid][8], sh[e] + 1);
+                store4(&sm.X[e * kBwdThreads + tid][12], sh[e] + 5);
+#pragma unroll
+                for (int i = 0; i < kHid / 2; ++i) u[e][i] = make_float2(sp[oB1 + 2 * i], sp[oB1 + 2 * i + 1]);
             }
 #pragma unroll
-            for (int q = 0; q < 2; ++q) store4(&sm.X[tid][8 + 4 * q], sh + 1 + 4 * q);
+            for (int k = 0; k < kSH; ++k) fma_pairs(sm.W1T[kFeat + k], sh[0][k], sh[1][k], u[0], u[1]);
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    *upad(sm, e * kBwdThreads + tid, q) = make_float4(u[e][2 * q].x, u[e][2 * q].y, u[e][2 * q + 1].x, u[e][2 * q + 1].y);
         }
+#pragma unroll 1
         for (int s = 0; s < t.S; ++s) {
-            // Rows are staged as soon as they are known; the ReLU masks of
-            // the hidden layers stay in registers as bits.
-            float d1[kHid], d3[4];
-            if (valid) {
-                float f[kFeat];
+            float d3[2][4];
 #pragma unroll
-                for (int c = 0; c < kFeat; ++c) f[c] = __ldg(V.feat + ((size_t)s * kFeat + c) * V.HW + p);
-                {
-                    const float x4[4] = {f[4], f[5], f[6], kC0};
-                    store4(&sm.X[tid][0], f);
-                    store4(&sm.X[tid][4], x4);
-                }
-                // Forward.  h1 as in the forward kernel; then each h2 unit in
-                // turn is staged and folded into the output accumulators, so
-                // that h2 never sits in registers as a whole (the same FMA
-                // order per output as the forward kernel).
-                unsigned m1 = 0, m2 = 0;
-                float h1[kHid];
+            for (int e = 0; e < 2; ++e) {
+                f[e][7] = kC0;
+                store4(&sm.X[e * kBwdThreads + tid][0], f[e]);
+                store4(&sm.X[e * kBwdThreads + tid][4], f[e] + 4);
+            }
+            // forward: rows are staged as soon as they are known
+            float2 h1[2][kHid / 2], h2[2][kHid / 2];
 #pragma unroll
-                for (int i = 0; i < kHid; ++i) {
-                    const float4 w0 = *reinterpret_cast<const float4*>(sp + oW1 + i * kIn);
-                    const float4 w1 = *reinterpret_cast<const float4*>(sp + oW1 + i * kIn + 4);
-                    float a = upad(sm, tid, i >> 2)[i & 3];
-                    a = fmaf(w0.x, f[0], a); a = fmaf(w0.y, f[1], a);
-                    a = fmaf(w0.z, f[2], a); a = fmaf(w0.w, f[3], a);
-                    a = fmaf(w1.x, f[4], a); a = fmaf(w1.y, f[5], a);
-                    a = fmaf(w1.z, f[6], a);
-                    h1[i] = fmaxf(a, 0.f);
-                    m1 |= (h1[i] > 0.f ? 1u : 0u) << i;
-                }
-#pragma unroll
-                for (int q = 0; q < 4; ++q) store4(&sm.H1[tid][4 * q], h1 + 4 * q);
-                float o[kOut];
-#pragma unroll
-                for (int c = 0; c < kOut; ++c) o[c] = sp[oB3 + c];
-#pragma unroll
-                for (int i = 0; i < kHid; ++i) {
-                    float a = sp[oB2 + i];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const float4 w = *reinterpret_cast<const float4*>(sp + oW2 + i * kHid + 4 * q);
-                        a = fmaf(w.x, h1[4 * q + 0], a); a = fmaf(w.y, h1[4 * q + 1], a);
-                        a = fmaf(w.z, h1[4 * q + 2], a); a = fmaf(w.w, h1[4 * q + 3], a);
-                    }
-                    const float h2 = fmaxf(a, 0.f);
-                    m2 |= (h2 > 0.f ? 1u : 0u) << i;
-                    sm.H2[tid][i] = h2;
-#pragma unroll
-                    for (int c = 0; c < kOut; ++c) o[c] = fmaf(sp[oW3 + c * kHid + i], h2, o[c]);
-                }
-#pragma unroll
-                for (int c = 0; c < kOut; ++c) o[c] = sigmoidf_(o[c]);
-                float g[kOut];
-#pragma unroll
-                for (int c = 0; c < kOut; ++c) g[c] = __ldcs(V.grad_rgb + ((size_t)s * kOut + c) * V.HW + p);
-                const float A = f[3];
-                float gA = 0.f;
-#pragma unroll
-                for (int c = 0; c < kOut; ++c) {
-                    gA = fmaf(g[c], f[c] - o[c], gA);
-                    const float go = (1.0f - A) * g[c];
-                    d3[c] = go * o[c] * (1.0f - o[c]);
-                }
-                d3[3] = 0.f;
-                // d2_j = (W3^T d3)_j [z2_j > 0], staged as soon as known and
-                // folded into d1 = W2^T d2 (then masked by [z1 > 0])
-#pragma unroll
-                for (int k = 0; k < kHid; ++k) d1[k] = 0.f;
-#pragma unroll
-                for (int j = 0; j < kHid; ++j) {
-                    float dj = 0.f;
-#pragma unroll
-                    for (int c = 0; c < kOut; ++c) dj = fmaf(sp[oW3 + c * kHid + j], d3[c], dj);
-                    dj = (m2 >> j) & 1u ? dj : 0.f;
-                    sm.D2[tid][j] = dj;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const float4 w = *reinterpret_cast<const float4*>(sp + oW2 + j * kHid + 4 * q);
-                        d1[4 * q + 0] = fmaf(w.x, dj, d1[4 * q + 0]); d1[4 * q + 1] = fmaf(w.y, dj, d1[4 * q + 1]);
-                        d1[4 * q + 2] = fmaf(w.z, dj, d1[4 * q + 2]); d1[4 * q + 3] = fmaf(w.w, dj, d1[4 * q + 3]);
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < kHid; ++k) d1[k] = (m1 >> k) & 1u ? d1[k] : 0.f;
-                // feature gradient: blend terms + (W1^T d1)[0:7]
-                if (V.grad_feat) {
-                    float gf[8];
-#pragma unroll
-                    for (int m = 0; m < 8; ++m) gf[m] = 0.f;
-#pragma unroll
-                    for (int k = 0; k < kHid; ++k) {
-                        const float4 w0 = *reinterpret_cast<const float4*>(sp + oW1 + k * kIn);
-                        const float4 w1 = *reinterpret_cast<const float4*>(sp + oW1 + k * kIn + 4);
-                        gf[0] = fmaf(w0.x, d1[k], gf[0]); gf[1] = fmaf(w0.y, d1[k], gf[1]);
-                        gf[2] = fmaf(w0.z, d1[k], gf[2]); gf[3] = fmaf(w0.w, d1[k], gf[3]);
-                        gf[4] = fmaf(w1.x, d1[k], gf[4]); gf[5] = fmaf(w1.y, d1[k], gf[5]);
-                        gf[6] = fmaf(w1.z, d1[k], gf[6]);
-                    }
-#pragma unroll
-                    for (int c = 0; c < kOut; ++c) gf[c] = fmaf(A, g[c], gf[c]);
-                    gf[3] += gA;
-                    float* dst = V.grad_feat + (size_t)s * kFeat * V.HW + p;
-                    if (t.overwrite) {
-#pragma unroll
-                        for (int c = 0; c < kFeat; ++c) dst[(size_t)c * V.HW] = gf[c];
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < kFeat; ++c) dst[(size_t)c * V.HW] += gf[c];
-                    }
-                }
-            } else {
-                const float z4[4] = {0.f, 0.f, 0.f, 0.f};
-                store4(&sm.X[tid][0], z4);
-                store4(&sm.X[tid][4], z4);
+            for (int e = 0; e < 2; ++e)
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    store4(&sm.H1[tid][4 * q], z4);
-                    store4(&sm.H2[tid][4 * q], z4);
+                    const float4 v = *upad(sm, e * kBwdThreads + tid, q);
+                    h1[e][2 * q] = make_float2(v.x, v.y);
+                    h1[e][2 * q + 1] = make_float2(v.z, v.w);
                 }
 #pragma unroll
-                for (int k = 0; k < kHid; ++k) d1[k] = 0.f;
+            for (int k = 0; k < kFeat; ++k) fma_pairs(sm.W1T[k], f[0][k], f[1][k], h1[0], h1[1]);
 #pragma unroll
-                for (int c = 0; c < 4; ++c) d3[c] = 0.f;
+            for (int e = 0; e < 2; ++e) {
 #pragma unroll
-                for (int q = 0; q < 4; ++q) store4(&sm.D2[tid][4 * q], z4);
+                for (int i = 0; i < kHid / 2; ++i) {
+                    h1[e][i] = make_float2(fmaxf(h1[e][i].x, 0.f), fmaxf(h1[e][i].y, 0.f));
+                    h2[e][i] = *reinterpret_cast<const float2*>(sp + oB2 + 2 * i);
+                }
+                store_pairs(sm.H1[e * kBwdThreads + tid], h1[e]);
             }
 #pragma unroll
-            for (int q = 0; q < 4; ++q) store4(&sm.D1[tid][4 * q], d1 + 4 * q);
-            store4(&sm.D3[tid][0], d3);
+            for (int k = 0; k < kHid; ++k) fma_pairs(sm.W2T[k], elem(h1[0], k), elem(h1[1], k), h2[0], h2[1]);
+            float o[2][kOut];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+#pragma unroll
+                for (int i = 0; i < kHid / 2; ++i) h2[e][i] = make_float2(fmaxf(h2[e][i].x, 0.f), fmaxf(h2[e][i].y, 0.f));
+                store_pairs(sm.H2[e * kBwdThreads + tid], h2[e]);
+#pragma unroll
+                for (int c = 0; c < kOut; ++c) o[e][c] = sp[oB3 + c];
+            }
+#pragma unroll
+            for (int i = 0; i < kHid; ++i) {
+                const float4 w = *reinterpret_cast<const float4*>(sm.W3T[i]);
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float h = elem(h2[e], i);
+                    o[e][0] = fmaf(w.x, h, o[e][0]);
+                    o[e][1] = fmaf(w.y, h, o[e][1]);
+                    o[e][2] = fmaf(w.z, h, o[e][2]);
+                }
+            }
+            float gA[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float A = f[e][3];
+                gA[e] = 0.f;
+#pragma unroll
+                for (int c = 0; c < kOut; ++c) {
+                    const float oc = sigmoidf_(o[e][c]);
+                    gA[e] = fmaf(g[e][c], f[e][c] - oc, gA[e]);
+                    const float go = (1.0f - A) * g[e][c];
+                    d3[e][c] = valid[e] ? go * oc * (1.0f - oc) : 0.f;
+                }
+                d3[e][3] = 0.f;
+                store4(sm.D3[e * kBwdThreads + tid], d3[e]);
+            }
+            // d2_j = (W3^T d3)_j [z2_j > 0]
+            float2 d2[2][kHid / 2] = {}, d1[2][kHid / 2] = {};
+#pragma unroll
+            for (int c = 0; c < kOut; ++c) fma_pairs(sp + oW3 + c * kHid, d3[0][c], d3[1][c], d2[0], d2[1]);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+#pragma unroll
+                for (int i = 0; i < kHid / 2; ++i)
+                    d2[e][i] = make_float2(h2[e][i].x > 0.f ? d2[e][i].x : 0.f, h2[e][i].y > 0.f ? d2[e][i].y : 0.f);
+                store_pairs(sm.D2[e * kBwdThreads + tid], d2[e]);
+            }
+            // d1 = (W2^T d2) [z1 > 0]
+#pragma unroll
+            for (int j = 0; j < kHid; ++j) fma_pairs(sp + oW2 + j * kHid, elem(d2[0], j), elem(d2[1], j), d1[0], d1[1]);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+#pragma unroll
+                for (int i = 0; i < kHid / 2; ++i)
+                    d1[e][i] = make_float2(h1[e][i].x > 0.f ? d1[e][i].x : 0.f, h1[e][i].y > 0.f ? d1[e][i].y : 0.f);
+                store_pairs(sm.D1[e * kBwdThreads + tid], d1[e]);
+            }
+            // feature gradient: blend terms + (W1^T d1)[0:7]
+            if (V.grad_feat) {
+                float2 gf[2][4] = {};
+#pragma unroll
+                for (int k = 0; k < kHid; ++k) fma_pairs(sp + oW1 + k * kIn, elem(d1[0], k), elem(d1[1], k), gf[0], gf[1]);
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    if (!valid[e]) continue;
+                    float* dst = V.grad_feat + (size_t)s * kFeat * V.HW + p[e];
+#pragma unroll
+                    for (int c = 0; c < kFeat; ++c) {
+                        float v = elem(gf[e], c);
+                        if (c < kOut) v = fmaf(f[e][3], g[e][c], v);
+                        if (c == 3) v += gA[e];
+                        if (t.overwrite) dst[(size_t)c * V.HW] = v;
+                        else dst[(size_t)c * V.HW] += v;
+                    }
+                }
+            }
+            // a pixel past the view's end adds nothing, whatever the weights are
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                if (valid[e]) continue;
+                const int r = e * kBwdThreads + tid;
+                for (int c = 0; c < kHid; ++c) sm.X[r][c] = sm.H1[r][c] = sm.H2[r][c] = sm.D1[r][c] = sm.D2[r][c] = 0.f;
+            }
+            if (s + 1 < t.S) load(b, s + 1);
+            else if (b + gridDim.x < t.n_blocks) load(b + gridDim.x, 0);
             __syncthreads();
             if (reducer) {
-                for (int q = grp; q < kThreads; q += kGroups) {
-                    const float4 d = *reinterpret_cast<const float4*>(Dsrc + q * dstride + 4 * ib);
-                    const float4 a = *reinterpret_cast<const float4*>(Asrc + q * kRow + 4 * jb);
-                    const float dv[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll 4
+                for (int q = grp; q < kPix; q += kGroups) {
+                    const float4 dv = *reinterpret_cast<const float4*>(Dsrc + q * kRow);
+                    const float4 aa = *reinterpret_cast<const float4*>(Asrc + q * kRow);
+                    const float4 ab = *reinterpret_cast<const float4*>(Asrc + q * kRow + 4);
+                    const float4 dz = *reinterpret_cast<const float4*>(sm.D3[q]);
+                    const float hz = sm.H2[q][blk];
+                    const float2 d[2] = {{dv.x, dv.y}, {dv.z, dv.w}}, sw[2] = {{dv.y, dv.x}, {dv.w, dv.z}};
+                    const float2 a[4] = {{aa.x, aa.y}, {aa.z, aa.w}, {ab.x, ab.y}, {ab.z, ab.w}};
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        acc[i][0] = fmaf(dv[i], a.x, acc[i][0]); acc[i][1] = fmaf(dv[i], a.y, acc[i][1]);
-                        acc[i][2] = fmaf(dv[i], a.z, acc[i][2]); acc[i][3] = fmaf(dv[i], a.w, acc[i][3]);
-                        accb[i] += dv[i];
+                    for (int i = 0; i < 2; ++i) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            accP[i][j] = __ffma2_rn(d[i], a[j], accP[i][j]);
+                            accQ[i][j] = __ffma2_rn(sw[i], a[j], accQ[i][j]);
+                        }
+                        accb[i] = __fadd2_rn(accb[i], d[i]);
                     }
+                    const float2 d01 = make_float2(dz.x, dz.y);
+                    acc3 = __ffma2_rn(d01, make_float2(hz, hz), acc3);
+                    acc3z = fmaf(dz.z, hz, acc3z);
+                    accb3 = __fadd2_rn(accb3, d01);
+                    accb3z += dz.z;
                 }
             }
             __syncthreads();
         }
     }
 
-    // Reduce the 7 pixel groups in shared memory, then one partial per CTA.
+    // Reduce the pixel groups in shared memory, then one partial per CTA.
     float* red = &sm.X[0][0];   // [kGroups][kParams]
-    for (int k = tid; k < kGroups * kParams; k += kThreads) red[k] = 0.f;
-    __syncthreads();
     if (reducer) {
         float* r = red + grp * kParams;
-        const int oW = layer == 0 ? oW1 : layer == 1 ? oW2 : oW3;
-        const int oB = layer == 0 ? oB1 : layer == 1 ? oB2 : oB3;
-        for (int i = 0; i < nrow; ++i) {
+        const int oW = layer == 0 ? oW1 : oW2, oB = layer == 0 ? oB1 : oB2;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
             const int row = 4 * ib + i;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) r[oW + row * kHid + 4 * jb + j] = acc[i][j];
-            if (bias_owner) r[oB + row] = accb[i];
+            for (int j = 0; j < 8; ++j) {
+                const float2 v = ((i ^ j) & 1) ? accQ[i >> 1][j >> 1] : accP[i >> 1][j >> 1];
+                r[oW + row * kHid + 8 * jb + j] = j & 1 ? v.y : v.x;
+            }
+            if (jb == 0) r[oB + row] = elem(accb, i);
+        }
+        r[oW3 + blk] = acc3.x;
+        r[oW3 + kHid + blk] = acc3.y;
+        r[oW3 + 2 * kHid + blk] = acc3z;
+        if (blk == 0) {
+            r[oB3] = accb3.x;
+            r[oB3 + 1] = accb3.y;
+            r[oB3 + 2] = accb3z;
         }
     }
     __syncthreads();
-    for (int k = tid; k < kParams; k += kThreads) {
+    for (int k = tid; k < kParams; k += kBwdThreads) {
         float a = 0.f;
 #pragma unroll
         for (int g = 0; g < kGroups; ++g) a += red[g * kParams + k];
@@ -777,7 +861,7 @@ int shade_bwd_grid() {
     int blocks = 0;
     const size_t smem = sizeof(BwdSmem);
     if (cudaFuncSetAttribute(k_shade_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_shade_bwd, kThreads, smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_shade_bwd, kBwdThreads, smem) != cudaSuccess ||
         blocks < 1) {
         cudaGetLastError();
         blocks = 1;
@@ -877,7 +961,7 @@ cudaError_t launch_shade_bwd(const ShadeView* views, int n, int S, const float* 
         cudaError_t e = cudaFuncSetAttribute(k_shade_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         const int g = grid < t.n_blocks ? grid : t.n_blocks;
-        k_shade_bwd<<<g, kThreads, smem, st>>>(t, params, partial);
+        k_shade_bwd<<<g, kBwdThreads, smem, st>>>(t, params, partial);
         note_launches(1);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if (grad_params) {
