@@ -26,11 +26,7 @@ __global__ void k_activate4(const float4* __restrict__ tex, float4* __restrict__
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n4; i += stride) {
         const float4 x = __ldg(tex + i);
-        float4 a;
-        a.x = pinned_sigmoid(x.x);
-        a.y = pinned_sigmoid(x.y);
-        a.z = pinned_sigmoid(x.z);
-        a.w = pinned_sigmoid(x.w);
+        const float4 a = pinned_sigmoid4(x);
         act[i] = a;
         const long long q = i / C4;
         if (i - q * C4 == C4 - 1) act_a[q] = a.w;

@@ -177,6 +177,34 @@ __device__ __forceinline__ float pinned_exp(float x) {
 // correctly rounded reciprocal is the IEEE division 1 / (1 + e^-x).
 __device__ __forceinline__ float pinned_sigmoid(float th) { return __frcp_rn(__fadd_rn(1.0f, pinned_exp(-th))); }
 
+// Four of them, the same bits: the range test and its branch once, e^-x as
+// packed pairs (the reduction and the polynomial of pinned_exp, each operation
+// with the same rounding).
+__device__ __forceinline__ float2 splat(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 exp_neg_near(float2 th) {   // e^-th, |th| < 80
+    const float2 x = make_float2(-th.x, -th.y);
+    const float2 m = __fadd2_rn(__fmul2_rn(x, splat(0x1.715476p+0f)), splat(0x1.8p+23f));
+    const float2 kf = __fadd2_rn(m, splat(-0x1.8p+23f));
+    const float2 r = __ffma2_rn(kf, splat(-0x1.7f7d1cp-20f), __ffma2_rn(kf, splat(-0x1.62e400p-1f), x));
+    float2 p = splat(0x1.a01a02p-13f);
+    p = __ffma2_rn(p, r, splat(0x1.6c16c2p-10f));
+    p = __ffma2_rn(p, r, splat(0x1.111112p-7f));
+    p = __ffma2_rn(p, r, splat(0x1.555556p-5f));
+    p = __ffma2_rn(p, r, splat(0x1.555556p-3f));
+    p = __ffma2_rn(p, r, splat(0.5f));
+    p = __ffma2_rn(p, r, splat(1.0f));
+    p = __ffma2_rn(p, r, splat(1.0f));
+    return __fmul2_rn(p, make_float2(__int_as_float((__float_as_int(m.x) + 127) << 23),
+                                     __int_as_float((__float_as_int(m.y) + 127) << 23)));
+}
+__device__ __forceinline__ float4 pinned_sigmoid4(float4 th) {
+    if (!(fabsf(th.x) < 80.0f && fabsf(th.y) < 80.0f && fabsf(th.z) < 80.0f && fabsf(th.w) < 80.0f))
+        return make_float4(pinned_sigmoid(th.x), pinned_sigmoid(th.y), pinned_sigmoid(th.z), pinned_sigmoid(th.w));
+    const float2 a = __fadd2_rn(splat(1.0f), exp_neg_near(make_float2(th.x, th.y)));
+    const float2 b = __fadd2_rn(splat(1.0f), exp_neg_near(make_float2(th.z, th.w)));
+    return make_float4(__frcp_rn(a.x), __frcp_rn(a.y), __frcp_rn(b.x), __frcp_rn(b.y));
+}
+
 // Philox4x32-10 block (Salmon et al., SC'11).
 __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1) {
 #pragma unroll
@@ -237,6 +265,11 @@ __device__ __forceinline__ Cell find_cell(int N, float b1, float b2) {
 
 __device__ __forceinline__ float interp(float a0, float a1, float a2, float wa, float wb) {
     return __fmaf_rn(wb, __fsub_rn(a2, a0), __fmaf_rn(wa, __fsub_rn(a1, a0), a0));
+}
+
+// The same for two channels, packed (a - b as fma(b, -1, a): one rounding).
+__device__ __forceinline__ float2 interp2(float2 a0, float2 a1, float2 a2, float2 wa, float2 wb) {
+    return __ffma2_rn(wb, __ffma2_rn(a0, splat(-1.0f), a2), __ffma2_rn(wa, __ffma2_rn(a0, splat(-1.0f), a1), a0));
 }
 
 // Pinned perspective-correct fragment from the three oriented (unbiased)
