@@ -389,7 +389,7 @@ __device__ __forceinline__ void winner_terms(const SoupDev& s, double* __restric
 }
 
 template <int SG, int TW>
-__global__ void __launch_bounds__(kTilePix, DS_MINB_BWD)
+__global__ void __launch_bounds__(kTilePix, SG == 4 ? DS_MINB_BWD4 : DS_MINB_BWD)
     k_raster_bwd(const __grid_constant__ ViewTable vt, const SoupDev s, const SetupRec* __restrict__ recs,
                  const uint32_t* __restrict__ keys, const uint32_t* __restrict__ vals,
                  const uint2* __restrict__ ranges, int DB, uint32_t flags, const GeomRec* __restrict__ geom,

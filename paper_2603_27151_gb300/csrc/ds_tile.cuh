@@ -12,7 +12,10 @@ constexpr unsigned kFullMask = 0xffffffffu;
 // Resident CTAs per SM requested from the compiler for the tile kernels
 // (register budget 65536 / (256 x blocks)); set per kernel at build time.
 // The backward and the fused training pass run at five (48 registers): their
-// waits on gathers hide better with 40 warps than the spills cost; the edge
+// waits on gathers hide better with 40 warps than the spills cost (847 against
+// 890 us for the backward of one sample, four 1080p views), but not in the
+// backward of four samples, whose spills are the largest (four 1080p and four
+// 960 x 540 views: 2755 us at five, 2686 at four); the edge
 // kernel and the forward of 4-sample groups are faster at four.  The
 // warp-sized forward runs at five with one sample (149 us against 159 at four
 // and 174 at six on 200,000 triangles at 1080p) and at four with two (78
@@ -28,6 +31,9 @@ constexpr unsigned kFullMask = 0xffffffffu;
 #endif
 #ifndef DS_MINB_BWD
 #define DS_MINB_BWD 5
+#endif
+#ifndef DS_MINB_BWD4
+#define DS_MINB_BWD4 4
 #endif
 #ifndef DS_MINB_EDGE
 #define DS_MINB_EDGE 4
