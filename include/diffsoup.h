@@ -557,7 +557,8 @@ DS_API ds_status ds_ctx_status(ds_ctx* ctx);
  * -1 = 16 (or fewer when the tile index needs the bits), 0 = unordered.
  * blocks_per_sm: CTAs per SM of the persistent tile kernels, 0 = each
  * kernel's occupancy limit.  chunk: triangles staged in shared memory per
- * round, a multiple of 32 in [32, 256].  Default {16, -1, 0, 256}. */
+ * round, a multiple of 32 in [32, 256] (forwards of one and two samples stage
+ * 32 per warp whatever it says).  Default {16, -1, 0, 256}. */
 typedef struct ds_tuning {
     int32_t tile_w, depth_bits, blocks_per_sm, chunk;
 } ds_tuning;
