@@ -10,6 +10,7 @@ from __future__ import annotations
 import ctypes
 import os
 import re
+import struct
 
 import numpy as np
 
@@ -209,8 +210,27 @@ def _stream(stream):
     return ctypes.c_void_p(stream.cuda_stream)
 
 
+# ds_camera in one write: 4 us per camera, all of them before a call's first
+# launch; a write per field took 9.
+_CAMERA = struct.Struct("=2i17f")
+
+
 def cameras(cams):
-    """Pack ``inputs.Camera`` objects into a ds_camera array."""
+    """Pack ``inputs.Camera`` objects into a ds_camera array: one write per
+    camera.  Values that do not fit int32 or float32 are converted field by
+    field, as ctypes does it."""
+    arr = (ds_camera * len(cams))()
+    try:
+        for k, c in enumerate(cams):
+            _CAMERA.pack_into(arr, k * _CAMERA.size, int(c.width), int(c.height), float(c.fx), float(c.fy), float(c.cx),
+                              float(c.cy), *np.asarray(c.R, np.float32).reshape(9).tolist(),
+                              *np.asarray(c.t, np.float32).reshape(3).tolist(), float(c.near))
+        return arr
+    except (OverflowError, struct.error):
+        return _cameras_by_field(cams)
+
+
+def _cameras_by_field(cams):
     arr = (ds_camera * len(cams))()
     for a, c in zip(arr, cams):
         a.width, a.height = int(c.width), int(c.height)
@@ -249,12 +269,11 @@ class Context:
         if S < 1:
             return   # the library rejects the sample count itself
 
-        def need(t, shape, dt, what):
-            if t is None:
+        def need(t, shape, dt, what, v=None):
+            if t is None or t.is_cuda and t.is_contiguous() and t.dtype == dt and (shape is None or t.shape == shape):
                 return
-            if not (t.is_cuda and t.is_contiguous() and t.dtype == dt and (shape is None or tuple(t.shape) == shape)):
-                raise ValueError("%s must be a contiguous %s CUDA tensor%s" % (what, dt, "" if shape is None else
-                                                                                " of shape %s" % (shape,)))
+            raise ValueError("%s%s must be a contiguous %s CUDA tensor%s" % (
+                what, "" if v is None else "[%d]" % v, dt, "" if shape is None else " of shape %s" % (shape,)))
         for name, lst in (("gbufs", gbufs), ("colors", colors), ("n_fronts", n_fronts), ("grad_colors", grad_colors),
                           ("score_ws", score_ws), ("targets", targets)):
             if lst is not None and len(lst) != n:
@@ -262,13 +281,18 @@ class Context:
         for v, (W, H) in enumerate(sizes):
             meta = self._soups.get(int(soup_ids[v]))
             Co = meta[1] - 1 if meta else None
-            need(gbufs[v] if gbufs is not None else None, (S, H, W, 4), torch.int32, "gbufs[%d]" % v)
-            need(n_fronts[v] if n_fronts is not None else None, (S, H, W), torch.int32, "n_fronts[%d]" % v)
-            need(score_ws[v] if score_ws is not None else None, (S, H, W), torch.float32, "score_ws[%d]" % v)
-            for name, lst, shape in (("colors", colors, (S, Co, H, W)), ("grad_colors", grad_colors, (S, Co, H, W)),
-                                     ("targets", targets, (Co, H, W))):
-                if lst is not None:
-                    need(lst[v], shape if meta else None, torch.float32, "%s[%d]" % (name, v))
+            if gbufs is not None:
+                need(gbufs[v], (S, H, W, 4), torch.int32, "gbufs", v)
+            if n_fronts is not None:
+                need(n_fronts[v], (S, H, W), torch.int32, "n_fronts", v)
+            if score_ws is not None:
+                need(score_ws[v], (S, H, W), torch.float32, "score_ws", v)
+            if colors is not None:
+                need(colors[v], (S, Co, H, W) if meta else None, torch.float32, "colors", v)
+            if grad_colors is not None:
+                need(grad_colors[v], (S, Co, H, W) if meta else None, torch.float32, "grad_colors", v)
+            if targets is not None:
+                need(targets[v], (Co, H, W) if meta else None, torch.float32, "targets", v)
         meta = self._soups.get(int(soup_ids[0])) if n else None
         if meta is not None:
             need(grad_verts, None, torch.float32, "grad_verts")
