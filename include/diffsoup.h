@@ -219,9 +219,10 @@ DS_API ds_status ds_raster_forward(ds_ctx* ctx, int32_t soup_id, const ds_camera
  * Score term: for every sample with weight w = score_w, +w/alpha for the
  * selected fragment and -w/(1-alpha) for every covered fragment in front of
  * it (all covered fragments when the sample shows the background), chained
- * to the opacity logits.  Contributions are summed in FP64 scratch with
- * atomics (summation order varies from run to run) and added to the FP32
- * outputs at the end. */
+ * to the opacity logits.  Contributions (FP32 sums over neighbouring lanes of
+ * a warp, the same groups in every run) are added up in FP64 scratch with
+ * atomics, whose order varies from run to run, and the result is added to the
+ * FP32 outputs. */
 DS_API ds_status ds_raster_backward(ds_ctx* ctx, int32_t soup_id, const ds_camera* cams,
                              int32_t n_views, int32_t S, const ds_view_out* fwd,
                              const ds_view_gin* gin, uint32_t grad_flags, float* grad_verts,
@@ -554,7 +555,8 @@ DS_API ds_status ds_ctx_status(ds_ctx* ctx);
  * result).  tile_w: tile width in pixels, 8, 16 or 32 (tiles hold 256 pixels,
  * so 8x32, 16x16 or 32x8).  depth_bits: bits of quantised nearest depth in
  * the bin key that order each tile's list front to back for the early exit,
- * -1 = 16 (or fewer when the tile index needs the bits), 0 = unordered.
+ * -1 = 16 (or fewer when the tile index needs the bits), 0 = none (lists in
+ * the order of the triangles).
  * blocks_per_sm: CTAs per SM of the persistent tile kernels, 0 = each
  * kernel's occupancy limit.  chunk: triangles staged in shared memory per
  * round, a multiple of 32 in [32, 256] (forwards of one and two samples stage

@@ -392,9 +392,9 @@ ds_status prepare(ds_ctx* c, int32_t plan_soup, Soup* const* soups, const ds_cam
                                 c->tcursor.as<uint32_t>(), c->keys[0].as<uint32_t>(), c->vals[0].as<uint32_t>(), limit,
                                 status, st);
         }
-        if (e != cudaSuccess || DB <= 0) return e;
+        if (e != cudaSuccess) return e;
         StageScope p(c, ds::kStSort, st);
-        return ds::launch_tile_sort(c->ranges.as<uint2>(), n_tiles, DB, c->keys[0].as<uint32_t>(),
+        return ds::launch_tile_sort(vt, c->ranges.as<uint2>(), n_tiles, DB, c->keys[0].as<uint32_t>(),
                                     c->vals[0].as<uint32_t>(), c->keys[1].as<uint32_t>(), c->vals[1].as<uint32_t>(), st);
     };
     DS_TRY_CUDA(offsets(cap));

@@ -1,12 +1,16 @@
 // ds_bin.cu -- binning of the set-up triangles into tiles: a counting sort by
-// tile, then (when the key has depth bits) a sort of each tile's list by depth.
+// tile, then a sort of each tile's list by (depth key, triangle).
 //
 // The set-up kernel counts the triangles of every tile (k_setup); the counts
 // are scanned over the tiles; k_emit places each (tile, triangle) pair at its
-// tile's cursor.  The order inside a tile's list does not matter for any
-// result (the depth test's tie-break is by triangle index), only for the early
-// exit of the walks, which wants the list front to back: k_tile_sort.  A
-// call makes 3-4 launches here.  The radix sort of (tile, depth) keys that
+// tile's cursor, in whatever order its atomics are served; k_tile_sort then
+// gives every list its one order.  The early exit of the walks wants it front
+// to back.  The triangle index breaks ties, and is the whole key when there
+// are no depth bits: the forward's results do not depend on the order (its
+// tie-break is by triangle index), but the backward sums the opacity terms of
+// neighbouring list entries in FP32 before the FP64 accumulators, and those
+// groups have to be the same in every call.  A call makes 4 launches here
+// (5 above 4,096 tiles) and a memset.  The radix sort of (tile, depth) keys that
 // this replaces made 4 passes of 5 launches over all pairs: 146 us of a
 // 1.28 ms training step (239,566 pairs), 39 us of a 120 us render of 64
 // triangles.
@@ -342,22 +346,23 @@ constexpr int kBlockList = 2048;    // up to this: the CTA, in shared memory; lo
 }  // namespace
 
 // Ranks of E entries per lane among the warp's n by counting the smaller ones
-// ((key, triangle) pairs are distinct), written back in order.
-template <int E>
+// ((key, triangle) pairs are distinct), written back in order; kKeys: there
+// are depth keys.
+template <int E, bool kKeys>
 __device__ __forceinline__ void sort_warp(uint32_t* keys, uint32_t* vals, uint32_t lo, int n, int lane) {
     uint32_t k[E], v[E];
     int rank[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         const bool in = lane + 32 * e < n;
-        k[e] = in ? keys[lo + lane + 32 * e] : 0u;
+        k[e] = kKeys && in ? keys[lo + lane + 32 * e] : 0u;
         v[e] = in ? vals[lo + lane + 32 * e] : 0u;
         rank[e] = 0;
     }
 #pragma unroll
     for (int f = 0; f < E; ++f)
         for (int j = 0; j < min(32, n - 32 * f); ++j) {
-            const uint32_t kj = __shfl_sync(kFull, k[f], j), vj = __shfl_sync(kFull, v[f], j);
+            const uint32_t kj = kKeys ? __shfl_sync(kFull, k[f], j) : 0u, vj = __shfl_sync(kFull, v[f], j);
 #pragma unroll
             for (int e = 0; e < E; ++e) rank[e] += kj < k[e] || (kj == k[e] && vj < v[e]) ? 1 : 0;
         }
@@ -365,18 +370,25 @@ __device__ __forceinline__ void sort_warp(uint32_t* keys, uint32_t* vals, uint32
 #pragma unroll
     for (int e = 0; e < E; ++e)
         if (lane + 32 * e < n) {
-            keys[lo + rank[e]] = k[e];
+            if (kKeys) keys[lo + rank[e]] = k[e];
             vals[lo + rank[e]] = v[e];
         }
 }
 
-// Every tile's list by depth key (front to back).  Most lists are short (a
+template <bool kKeys>
+__device__ __forceinline__ void sort_short(uint32_t* keys, uint32_t* vals, uint32_t lo, int n, int lane) {
+    if (n > 64) sort_warp<4, kKeys>(keys, vals, lo, n, lane);
+    else if (n > 32) sort_warp<2, kKeys>(keys, vals, lo, n, lane);
+    else if (n > 1) sort_warp<1, kKeys>(keys, vals, lo, n, lane);
+}
+
+// Every tile's list by (depth key, triangle).  Most lists are short (a
 // few dozen triangles): one warp each.  The CTA then takes its tiles with
 // long lists one after the other: up to kBlockList entries by a bitonic
 // network in shared memory, longer ones by stable 8-bit LSD passes between
-// the two buffers.  A CTA's tiles are gridDim.x apart, since long lists come
-// in neighbouring tiles.
-__global__ void __launch_bounds__(256) k_tile_sort(const uint2* __restrict__ ranges, int n_tiles, int DB,
+// the two buffers, the triangle's digits (tri_passes) first.  A CTA's tiles
+// are gridDim.x apart, since long lists come in neighbouring tiles.
+__global__ void __launch_bounds__(256) k_tile_sort(const uint2* __restrict__ ranges, int n_tiles, int DB, int tri_passes,
                                                    uint32_t* __restrict__ k0, uint32_t* __restrict__ v0,
                                                    uint32_t* __restrict__ k1, uint32_t* __restrict__ v1) {
     __shared__ unsigned long long s_kv[kBlockList];
@@ -388,9 +400,8 @@ __global__ void __launch_bounds__(256) k_tile_sort(const uint2* __restrict__ ran
         const uint2 rg = ranges[blockIdx.x + warp * gridDim.x];
         const int n = (int)(rg.y - rg.x);
         if (n > kWarpList) lng = true;
-        else if (n > 64) sort_warp<4>(k0, v0, rg.x, n, lane);
-        else if (n > 32) sort_warp<2>(k0, v0, rg.x, n, lane);
-        else if (n > 1) sort_warp<1>(k0, v0, rg.x, n, lane);
+        else if (DB > 0) sort_short<true>(k0, v0, rg.x, n, lane);
+        else sort_short<false>(k0, v0, rg.x, n, lane);
     }
     if (!__syncthreads_or(lng)) return;
     for (int q = 0; q < kSortWarps; ++q) {
@@ -403,7 +414,7 @@ __global__ void __launch_bounds__(256) k_tile_sort(const uint2* __restrict__ ran
             int m = 256;
             while (m < n) m <<= 1;
             for (int i = tid; i < m; i += 256)
-                s_kv[i] = i < n ? ((unsigned long long)k0[rg.x + i] << 32) | v0[rg.x + i] : ~0ull;
+                s_kv[i] = i < n ? ((unsigned long long)(DB > 0 ? k0[rg.x + i] : 0u) << 32) | v0[rg.x + i] : ~0ull;
             for (int k = 2; k <= m; k <<= 1)
                 for (int j = k >> 1; j > 0; j >>= 1) {
                     __syncthreads();
@@ -418,17 +429,19 @@ __global__ void __launch_bounds__(256) k_tile_sort(const uint2* __restrict__ ran
                 }
             __syncthreads();
             for (int i = tid; i < n; i += 256) {
-                k0[rg.x + i] = (uint32_t)(s_kv[i] >> 32);
+                if (DB > 0) k0[rg.x + i] = (uint32_t)(s_kv[i] >> 32);
                 v0[rg.x + i] = (uint32_t)s_kv[i];
             }
             continue;
         }
         uint32_t *ki = k0, *vi = v0, *ko = k1, *vo = v1;
         const unsigned lt = (1u << lane) - 1u;
-        for (int shift = 0; shift < DB; shift += 8) {
+        for (int pass = 0; pass < tri_passes + (DB + 7) / 8; ++pass) {
+            const bool by_tri = pass < tri_passes;
+            const int shift = 8 * (by_tri ? pass : pass - tri_passes);
             s_base[tid] = 0;
             __syncthreads();
-            for (uint32_t i = rg.x + tid; i < rg.y; i += 256) atomicAdd(&s_base[(ki[i] >> shift) & 255u], 1u);
+            for (uint32_t i = rg.x + tid; i < rg.y; i += 256) atomicAdd(&s_base[((by_tri ? vi[i] : ki[i]) >> shift) & 255u], 1u);
             __syncthreads();
             // exclusive scan of the 256 digit counts
             const uint32_t c = s_base[tid];
@@ -450,8 +463,8 @@ __global__ void __launch_bounds__(256) k_tile_sort(const uint2* __restrict__ ran
                 __syncthreads();
                 const uint32_t i = i0 + tid;
                 const bool in = i < rg.y;
-                const uint32_t key = in ? ki[i] : 0u, val = in ? vi[i] : 0u;
-                const uint32_t d = in ? ((key >> shift) & 255u) : 256u;
+                const uint32_t key = DB > 0 && in ? ki[i] : 0u, val = in ? vi[i] : 0u;
+                const uint32_t d = in ? (((by_tri ? val : key) >> shift) & 255u) : 256u;
                 const unsigned peers = __match_any_sync(kFull, d);
                 const uint32_t wrank = __popc(peers & lt);
                 if (in && wrank == 0) s_w[warp][d] = __popc(peers);
@@ -469,7 +482,7 @@ __global__ void __launch_bounds__(256) k_tile_sort(const uint2* __restrict__ ran
                 __syncthreads();
                 if (in) {
                     const uint32_t pos = rg.x + s_w[warp][d] + wrank;
-                    ko[pos] = key;
+                    if (DB > 0) ko[pos] = key;
                     vo[pos] = val;
                 }
                 __syncthreads();
@@ -481,19 +494,21 @@ __global__ void __launch_bounds__(256) k_tile_sort(const uint2* __restrict__ ran
             vi = vo;
             vo = x;
         }
-        if (ki != k0)
+        if (vi != v0)
             for (uint32_t i = rg.x + tid; i < rg.y; i += 256) {
-                k0[i] = ki[i];
+                if (DB > 0) k0[i] = ki[i];
                 v0[i] = vi[i];
             }
         __syncthreads();
     }
 }
 
-cudaError_t launch_tile_sort(const uint2* ranges, int n_tiles, int DB, uint32_t* k0, uint32_t* v0, uint32_t* k1,
-                             uint32_t* v1, cudaStream_t st) {
-    if (DB <= 0) return cudaSuccess;
-    k_tile_sort<<<(n_tiles + kSortWarps - 1) / kSortWarps, 256, 0, st>>>(ranges, n_tiles, DB, k0, v0, k1, v1);
+cudaError_t launch_tile_sort(const ViewTable& vt, const uint2* ranges, int n_tiles, int DB, uint32_t* k0, uint32_t* v0,
+                             uint32_t* k1, uint32_t* v1, cudaStream_t st) {
+    int tri_passes = 1;   // 8-bit digits of the largest triangle index
+    for (int v = 0; v < vt.n; ++v)
+        while (vt.v[v].s_T > 1 << 8 * tri_passes) ++tri_passes;
+    k_tile_sort<<<(n_tiles + kSortWarps - 1) / kSortWarps, 256, 0, st>>>(ranges, n_tiles, DB, tri_passes, k0, v0, k1, v1);
     note_launches(1);
     return cudaGetLastError();
 }

@@ -62,9 +62,9 @@ cudaError_t launch_tile_offsets(const uint32_t* count, int n_tiles, uint32_t cap
 // (if status is not NULL).
 cudaError_t launch_emit(const ViewTable& vt, const SetupRec* recs, const int4* tbox, const uint32_t* zkeys, int DB,
                         uint32_t* cursor, uint32_t* keys, uint32_t* vals, uint32_t cap, int* status, cudaStream_t st);
-// The lists front to back (nothing to do when DB = 0); k1, v1: scratch of the
-// lists' size.
-cudaError_t launch_tile_sort(const uint2* ranges, int n_tiles, int DB, uint32_t* k0, uint32_t* v0, uint32_t* k1,
+// Every list by (depth key, triangle), by triangle when DB = 0; k1, v1: scratch
+// of the lists' size.
+cudaError_t launch_tile_sort(const ViewTable& vt, const uint2* ranges, int n_tiles, int DB, uint32_t* k0, uint32_t* v0, uint32_t* k1,
                              uint32_t* v1, cudaStream_t st);
 
 // ---- forward rasteriser (ds_raster.cu)

@@ -176,7 +176,7 @@ extern "C" DS_API ds_status ds_raster_forward_noalloc(const float* verts, const 
     while (tile_bits < 32 && (1ull << tile_bits) < (unsigned long long)tile_base) ++tile_bits;
     const int DB = tile_bits <= 16 ? 16 : 32 - tile_bits;
     NA_TRY(ds::launch_emit(vt, recs, tbox, zkeys, DB, tcursor, keys[0], vals[0], (uint32_t)kMaxPairs, status, st));
-    NA_TRY(ds::launch_tile_sort(ranges, tile_base, DB, keys[0], vals[0], keys[1], vals[1], st));
+    NA_TRY(ds::launch_tile_sort(vt, ranges, tile_base, DB, keys[0], vals[0], keys[1], vals[1], st));
     ds::Bg b{};
     for (int i = 0; i < C - 1; ++i) b.c[i] = bg[i];
     const int grid = 0;
