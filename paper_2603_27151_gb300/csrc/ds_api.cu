@@ -109,7 +109,7 @@ struct ds_ctx {
     int device = 0;
     std::mutex mu;
     std::vector<Soup> soups;
-    DevBuf recs, tbox, zkeys, keys[2], vals[2], tcount, tcursor, tsums, ranges, misc, geom;
+    DevBuf recs, tbox, zkeys, keys[2], vals[2], chunks, tcount, tcursor, tsums, ranges, misc, geom;
     DevBuf acc_tex, acc_verts;   // FP64 gradient accumulators of the backward
     DevBuf shade_part;           // per-CTA partials of the shading parameter gradients
     DevBuf plan_dev;             // device copy of an adaptive-control plan
@@ -136,6 +136,7 @@ struct ds_ctx {
     // misc layout (work counters: 0 forward, 1 and 4 counts, 2 backward, 3 edges)
     int* d_status() const { return misc.as<int>(); }
     int* d_counter() const { return misc.as<int>() + 4; }
+    // pairs of the lists, chunks of the long ones
     uint32_t* d_K() const { return reinterpret_cast<uint32_t*>(misc.as<int>() + 12); }
     unsigned long long* d_total() const { return reinterpret_cast<unsigned long long*>(misc.as<char>() + 64); }
 };
@@ -148,6 +149,15 @@ constexpr int kCounters = 5;
 uint32_t pair_capacity(const ds_ctx* c) {
     size_t n = std::min(std::min(c->keys[0].cap, c->keys[1].cap), std::min(c->vals[0].cap, c->vals[1].cap)) / 4;
     return (uint32_t)std::min<size_t>(n, 0xffffffffu);
+}
+
+// List buffers for at least K pairs.
+ds_status ensure_pairs(ds_ctx* c, size_t K) {
+    for (int b = 0; b < 2; ++b) {
+        DS_TRY(c->keys[b].ensure(4 * K, "bin keys"));
+        DS_TRY(c->vals[b].ensure(4 * K, "bin values"));
+    }
+    return c->chunks.ensure(sizeof(uint2) * ds::max_chunks(pair_capacity(c)), "list chunks");
 }
 
 struct DeviceGuard {
@@ -381,8 +391,8 @@ ds_status prepare(ds_ctx* c, int32_t plan_soup, Soup* const* soups, const ds_cam
     auto offsets = [&](uint32_t limit) {
         StageScope p(c, ds::kStScan, st);
         return ds::launch_tile_offsets(c->tcount.as<uint32_t>(), n_tiles, limit, c->tsums.as<uint32_t>(),
-                                       c->ranges.as<uint2>(), c->tcursor.as<uint32_t>(), c->d_K(), c->d_counter(),
-                                       kCounters, st);
+                                       c->ranges.as<uint2>(), c->tcursor.as<uint32_t>(), c->d_K(), c->chunks.as<uint2>(),
+                                       c->d_counter(), kCounters, st);
     };
     auto lists = [&](uint32_t limit, int* status) {
         cudaError_t e = cudaSuccess;
@@ -394,30 +404,43 @@ ds_status prepare(ds_ctx* c, int32_t plan_soup, Soup* const* soups, const ds_cam
         }
         if (e != cudaSuccess) return e;
         StageScope p(c, ds::kStSort, st);
-        return ds::launch_tile_sort(vt, c->ranges.as<uint2>(), n_tiles, DB, c->keys[0].as<uint32_t>(),
-                                    c->vals[0].as<uint32_t>(), c->keys[1].as<uint32_t>(), c->vals[1].as<uint32_t>(), st);
+        return ds::launch_tile_sort(vt, c->ranges.as<uint2>(), n_tiles, DB, c->d_K() + 1, c->chunks.as<uint2>(), limit,
+                                    c->keys[0].as<uint32_t>(), c->vals[0].as<uint32_t>(), c->keys[1].as<uint32_t>(),
+                                    c->vals[1].as<uint32_t>(), st);
+    };
+    auto merge = [&](uint32_t limit) {
+        StageScope p(c, ds::kStSort, st);
+        return ds::launch_list_merge(c->ranges.as<uint2>(), DB, c->d_K() + 1, c->chunks.as<uint2>(), limit,
+                                     c->keys[0].as<uint32_t>(), c->vals[0].as<uint32_t>(), c->keys[1].as<uint32_t>(),
+                                     c->vals[1].as<uint32_t>(), st);
     };
     DS_TRY_CUDA(offsets(cap));
     // With a host wait for the number of pairs: the lists are built with the
     // buffers there are while the number travels, and built again if they
-    // turn out to be too small.
+    // turn out to be too small.  The number of long lists' chunks comes with
+    // it, so that the merge is launched when there are some; without the wait
+    // it is launched when there can be.
     if (wait) {
-        DS_TRY_CUDA(cudaMemcpyAsync(c->h_word, c->d_K(), 4, cudaMemcpyDeviceToHost, st));
+        DS_TRY_CUDA(cudaMemcpyAsync(c->h_word, c->d_K(), 8, cudaMemcpyDeviceToHost, st));
         DS_TRY_CUDA(cudaEventRecord(c->k_event, st));
     }
     if (cap > 0) DS_TRY_CUDA(lists(cap, wait ? nullptr : c->d_status()));
+    bool merge_lists = ds::long_lists(vt);
     if (wait) {
         DS_TRY_CUDA(cudaEventSynchronize(c->k_event));
-        const uint32_t K = *c->h_word;
+        const uint32_t K = c->h_word[0];
         if (K > cap || cap == 0) {
-            for (int b = 0; b < 2; ++b) {
-                DS_TRY(c->keys[b].ensure(4 * (size_t)(K > 0 ? K : 1), "bin keys"));
-                DS_TRY(c->vals[b].ensure(4 * (size_t)(K > 0 ? K : 1), "bin values"));
-            }
-            DS_TRY_CUDA(offsets(pair_capacity(c)));
-            DS_TRY_CUDA(lists(pair_capacity(c), nullptr));
+            DS_TRY(ensure_pairs(c, K > 0 ? K : 1));
+            cap = pair_capacity(c);
+            DS_TRY_CUDA(offsets(cap));
+            DS_TRY_CUDA(lists(cap, nullptr));
+        } else {
+            merge_lists = merge_lists && c->h_word[1] > 0;
         }
+        if (merge_lists) DS_TRY_CUDA(merge(cap));
         cap = K;
+    } else if (merge_lists) {
+        DS_TRY_CUDA(merge(cap));
     }
 
     c->plan.valid = true;
@@ -507,7 +530,7 @@ void ds_destroy(ds_ctx* c) {
         if (s.act) cudaFree(s.act);
     }
     DevBuf* bufs[] = {&c->recs, &c->tbox, &c->zkeys, &c->keys[0], &c->keys[1], &c->vals[0], &c->vals[1],
-                      &c->tcount, &c->tcursor, &c->tsums, &c->ranges, &c->misc, &c->geom, &c->acc_tex, &c->acc_verts, &c->shade_part, &c->plan_dev};
+                      &c->chunks, &c->tcount, &c->tcursor, &c->tsums, &c->ranges, &c->misc, &c->geom, &c->acc_tex, &c->acc_verts, &c->shade_part, &c->plan_dev};
     for (DevBuf* b : bufs) b->release();
     if (c->h_word) cudaFreeHost(c->h_word);
     if (c->k_event) cudaEventDestroy(c->k_event);
@@ -1018,12 +1041,7 @@ ds_status ds_reserve(ds_ctx* c, int64_t pairs) {
     if (!c || pairs < 0 || pairs > 0x7fffffffLL) return fail(DS_ERR_INVALID_ARG, "bad context or pair count");
     std::lock_guard<std::mutex> lk(c->mu);
     DeviceGuard g(c->device);
-    const size_t K = (size_t)(pairs > 0 ? pairs : 1);
-    for (int b = 0; b < 2; ++b) {
-        DS_TRY(c->keys[b].ensure(4 * K, "bin keys"));
-        DS_TRY(c->vals[b].ensure(4 * K, "bin values"));
-    }
-    return DS_OK;
+    return ensure_pairs(c, (size_t)(pairs > 0 ? pairs : 1));
 }
 
 ds_status ds_fragment_count(ds_ctx* c, int32_t soup_id, const ds_camera* cams, int32_t n_views,

@@ -4,7 +4,8 @@
 // The set-up kernel counts the triangles of every tile (k_setup); the counts
 // are scanned over the tiles; k_emit places each (tile, triangle) pair at its
 // tile's cursor, in whatever order its atomics are served; k_tile_sort then
-// gives every list its one order.  The early exit of the walks wants it front
+// (with k_list_merge for lists above 2,048 entries) gives every list its one
+// order.  The early exit of the walks wants it front
 // to back.  The triangle index breaks ties, and is the whole key when there
 // are no depth bits: the forward's results do not depend on the order (its
 // tie-break is by triangle index), but the backward sums the opacity terms of
@@ -14,6 +15,8 @@
 // this replaces made 4 passes of 5 launches over all pairs: 146 us of a
 // 1.28 ms training step (239,566 pairs), 39 us of a 120 us render of 64
 // triangles.
+#include <algorithm>
+
 #include "ds_internal.h"
 
 namespace ds {
@@ -223,10 +226,11 @@ cudaError_t launch_setup(const ViewTable& vt, int n_tiles, SetupRec* recs, uint3
 // ---------------------------------------------------------------- tile offsets
 // Sum of one block's kScanBlock tile counts (1024 threads x 4).
 __global__ void __launch_bounds__(1024) k_tile_sums(const uint32_t* __restrict__ count, int n,
-                                                    uint32_t* __restrict__ block_sum) {
+                                                    uint32_t* __restrict__ block_sum, uint32_t* __restrict__ total) {
     __shared__ uint32_t wsum[32];
     const int tid = threadIdx.x, base = blockIdx.x * kScanBlock + 4 * tid;
     uint32_t s = 0;
+    if (blockIdx.x == 0 && tid == 0) total[1] = 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) s += base + k < n ? count[base + k] : 0u;
     s = __reduce_add_sync(kFull, s);
@@ -239,15 +243,18 @@ __global__ void __launch_bounds__(1024) k_tile_sums(const uint32_t* __restrict__
 }
 
 // Exclusive scan of the tile counts: every tile's range in the lists (cut at
-// the capacity `cap`) and its cursor for k_emit, the number of pairs, and
-// the tile kernels' work counters set to zero.  Block b adds up the sums of the
-// blocks before it itself (at most 4,096 for the largest call).
+// the capacity `cap`) and its cursor for k_emit, the number of pairs total[0],
+// the chunks of the lists above kBlockList entries and their number total[1],
+// and the tile kernels' work counters set to zero.  Block b adds up the sums of
+// the blocks before it itself (at most 4,096 for the largest call).
 __global__ void __launch_bounds__(1024) k_tile_offsets(const uint32_t* __restrict__ count, int n, uint32_t cap,
                                                        const uint32_t* __restrict__ block_sum, uint2* __restrict__ ranges,
                                                        uint32_t* __restrict__ cursor, uint32_t* __restrict__ total,
-                                                       int* __restrict__ counters, int n_counters) {
+                                                       uint2* __restrict__ chunks, int* __restrict__ counters,
+                                                       int n_counters) {
     __shared__ uint32_t wsum[32], wpre[32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, base = blockIdx.x * kScanBlock + 4 * tid;
+    if (gridDim.x == 1 && tid == 0) total[1] = 0;   // else k_tile_sums has cleared it
     uint32_t before = 0;
     for (int b = tid; b < (int)blockIdx.x; b += 1024) before += block_sum[b];
     before = __reduce_add_sync(kFull, before);
@@ -271,8 +278,13 @@ __global__ void __launch_bounds__(1024) k_tile_offsets(const uint32_t* __restric
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         if (base + k < n) {
-            ranges[base + k] = make_uint2(min(off, cap), min(off + x[k], cap));
+            const uint32_t lo = min(off, cap), hi = min(off + x[k], cap);
+            ranges[base + k] = make_uint2(lo, hi);
             cursor[base + k] = off;
+            if (hi - lo > kBlockList) {
+                const uint32_t m = (hi - lo + kBlockList - 1) / kBlockList, at = atomicAdd(total + 1, m);
+                for (uint32_t c = 0; c < m; ++c) chunks[at + c] = make_uint2((uint32_t)(base + k), c);
+            }
             if (base + k == n - 1) *total = off + x[k];
         }
         off += x[k];
@@ -281,13 +293,15 @@ __global__ void __launch_bounds__(1024) k_tile_offsets(const uint32_t* __restric
 }
 
 cudaError_t launch_tile_offsets(const uint32_t* count, int n_tiles, uint32_t cap, uint32_t* block_sum, uint2* ranges,
-                                uint32_t* cursor, uint32_t* total, int* counters, int n_counters, cudaStream_t st) {
+                                uint32_t* cursor, uint32_t* total, uint2* chunks, int* counters, int n_counters,
+                                cudaStream_t st) {
     const int nblk = (n_tiles + kScanBlock - 1) / kScanBlock;
     if (nblk > 1) {
-        k_tile_sums<<<nblk, 1024, 0, st>>>(count, n_tiles, block_sum);
+        k_tile_sums<<<nblk, 1024, 0, st>>>(count, n_tiles, block_sum, total);
         note_launches(1);
     }
-    k_tile_offsets<<<nblk, 1024, 0, st>>>(count, n_tiles, cap, block_sum, ranges, cursor, total, counters, n_counters);
+    k_tile_offsets<<<nblk, 1024, 0, st>>>(count, n_tiles, cap, block_sum, ranges, cursor, total, chunks, counters,
+                                             n_counters);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -339,10 +353,13 @@ cudaError_t launch_emit(const ViewTable& vt, const SetupRec* recs, const int4* t
 }
 
 // ---------------------------------------------------------------- depth order
+// Sort times below in us: (a) 100,000 triangles in eight 1080p views, (b)
+// 2,000 and (c) 20,000 in a 64 x 64 view (16 lists), (d) 200,000 there with
+// lists of 13,000, (e) 1,000,000 there with lists of 45,000, 16 depth bits.
 namespace {
-constexpr int kSortWarps = 8;       // tiles per CTA of k_tile_sort
-constexpr int kWarpList = 128;      // lists up to this length: one warp, in registers
-constexpr int kBlockList = 2048;    // up to this: the CTA, in shared memory; longer: radix passes in global memory
+constexpr int kSortWarps = 8;       // most tiles per CTA of k_tile_sort
+constexpr int kWarpList = 128;      // lists up to this length: one warp, in registers (64: a 76 -> 109, b 24 -> 11)
+constexpr int kSortThreads = 256;   // 512: a 76 -> 99, d 51 -> 45
 }  // namespace
 
 // Ranks of E entries per lane among the warp's n by counting the smaller ones
@@ -382,133 +399,156 @@ __device__ __forceinline__ void sort_short(uint32_t* keys, uint32_t* vals, uint3
     else if (n > 1) sort_warp<1, kKeys>(keys, vals, lo, n, lane);
 }
 
-// Every tile's list by (depth key, triangle).  Most lists are short (a
-// few dozen triangles): one warp each.  The CTA then takes its tiles with
-// long lists one after the other: up to kBlockList entries by a bitonic
-// network in shared memory, longer ones by stable 8-bit LSD passes between
-// the two buffers, the triangle's digits (tri_passes) first.  A CTA's tiles
-// are gridDim.x apart, since long lists come in neighbouring tiles.
-__global__ void __launch_bounds__(256) k_tile_sort(const uint2* __restrict__ ranges, int n_tiles, int DB, int tri_passes,
-                                                   uint32_t* __restrict__ k0, uint32_t* __restrict__ v0,
-                                                   uint32_t* __restrict__ k1, uint32_t* __restrict__ v1) {
+// n <= kBlockList entries (depth key, triangle) from k, v in order into ko, vo
+// (which may be k and v): a bitonic network in shared memory.
+__device__ __forceinline__ void sort_block(unsigned long long* s_kv, const uint32_t* k, const uint32_t* v, uint32_t* ko,
+                                           uint32_t* vo, int n, bool keys) {
+    const int tid = threadIdx.x;
+    int m = kSortThreads;
+    while (m < n) m <<= 1;
+    for (int i = tid; i < m; i += kSortThreads)
+        s_kv[i] = i < n ? ((unsigned long long)(keys ? k[i] : 0u) << 32) | v[i] : ~0ull;
+    for (int w = 2; w <= m; w <<= 1)
+        for (int j = w >> 1; j > 0; j >>= 1) {
+            __syncthreads();
+            for (int p = tid; p < m / 2; p += kSortThreads) {
+                const int i = 2 * p - (p & (j - 1));   // the pair (i, i + j)
+                const unsigned long long a = s_kv[i], b = s_kv[i + j];
+                if ((a > b) == ((i & w) == 0)) {
+                    s_kv[i] = b;
+                    s_kv[i + j] = a;
+                }
+            }
+        }
+    __syncthreads();
+    for (int i = tid; i < n; i += kSortThreads) {
+        if (keys) ko[i] = (uint32_t)(s_kv[i] >> 32);
+        vo[i] = (uint32_t)s_kv[i];
+    }
+    __syncthreads();
+}
+
+// Every tile's list by (depth key, triangle).  Most lists are short (a few
+// dozen triangles): one warp each.  The CTA then takes its tiles with lists
+// above kWarpList one after the other, and of the lists above kBlockList its
+// share of the chunks, which go to (k1, v1) for k_list_merge.  A CTA's `per`
+// tiles are gridDim.x apart, since long lists come in neighbouring tiles.
+// Bound by the latency of the network's stages (c) or by shared memory (e).
+// With eight tiles to every CTA and lists above 2,048 entries in radix passes
+// of one CTA: b 49, c 137, d 582, e 2,029 us; now 24, 51, 51 and 132 (a global
+// radix sort of all pairs: 64, 80, 109 and 117, and a 171 against 76).
+__global__ void __launch_bounds__(kSortThreads) k_tile_sort(const uint2* __restrict__ ranges, int n_tiles, int per, int DB,
+                                                            const uint32_t* __restrict__ n_chunks,
+                                                            const uint2* __restrict__ chunks, uint32_t* __restrict__ k0,
+                                                            uint32_t* __restrict__ v0, uint32_t* __restrict__ k1,
+                                                            uint32_t* __restrict__ v1) {
     __shared__ unsigned long long s_kv[kBlockList];
-    __shared__ uint32_t s_base[256], s_w[kSortWarps][256];
-    __shared__ uint32_t s_tot[kSortWarps];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     bool lng = false;
-    if ((int)(blockIdx.x + warp * gridDim.x) < n_tiles) {
-        const uint2 rg = ranges[blockIdx.x + warp * gridDim.x];
+    const int tile = blockIdx.x + warp * gridDim.x;
+    if (warp < per && tile < n_tiles) {
+        const uint2 rg = ranges[tile];
         const int n = (int)(rg.y - rg.x);
         if (n > kWarpList) lng = true;
         else if (DB > 0) sort_short<true>(k0, v0, rg.x, n, lane);
         else sort_short<false>(k0, v0, rg.x, n, lane);
     }
-    if (!__syncthreads_or(lng)) return;
-    for (int q = 0; q < kSortWarps; ++q) {
+    const bool any = __syncthreads_or(lng);
+    for (int q = 0; any && q < per; ++q) {
         if ((int)(blockIdx.x + q * gridDim.x) >= n_tiles) break;
         const uint2 rg = ranges[blockIdx.x + q * gridDim.x];
         const int n = (int)(rg.y - rg.x);
-        if (n <= kWarpList) continue;
-        __syncthreads();
-        if (n <= kBlockList) {
-            int m = 256;
-            while (m < n) m <<= 1;
-            for (int i = tid; i < m; i += 256)
-                s_kv[i] = i < n ? ((unsigned long long)(DB > 0 ? k0[rg.x + i] : 0u) << 32) | v0[rg.x + i] : ~0ull;
-            for (int k = 2; k <= m; k <<= 1)
-                for (int j = k >> 1; j > 0; j >>= 1) {
-                    __syncthreads();
-                    for (int p = tid; p < m / 2; p += 256) {
-                        const int i = 2 * p - (p & (j - 1));   // the pair (i, i + j)
-                        const unsigned long long a = s_kv[i], b = s_kv[i + j];
-                        if ((a > b) == ((i & k) == 0)) {
-                            s_kv[i] = b;
-                            s_kv[i + j] = a;
-                        }
-                    }
-                }
-            __syncthreads();
-            for (int i = tid; i < n; i += 256) {
-                if (DB > 0) k0[rg.x + i] = (uint32_t)(s_kv[i] >> 32);
-                v0[rg.x + i] = (uint32_t)s_kv[i];
-            }
-            continue;
-        }
-        uint32_t *ki = k0, *vi = v0, *ko = k1, *vo = v1;
-        const unsigned lt = (1u << lane) - 1u;
-        for (int pass = 0; pass < tri_passes + (DB + 7) / 8; ++pass) {
-            const bool by_tri = pass < tri_passes;
-            const int shift = 8 * (by_tri ? pass : pass - tri_passes);
-            s_base[tid] = 0;
-            __syncthreads();
-            for (uint32_t i = rg.x + tid; i < rg.y; i += 256) atomicAdd(&s_base[((by_tri ? vi[i] : ki[i]) >> shift) & 255u], 1u);
-            __syncthreads();
-            // exclusive scan of the 256 digit counts
-            const uint32_t c = s_base[tid];
-            uint32_t inc = c;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const uint32_t o = __shfl_up_sync(kFull, inc, d);
-                if (lane >= d) inc += o;
-            }
-            if (lane == 31) s_tot[warp] = inc;
-            __syncthreads();
-            uint32_t pre = inc - c;
-            for (int w = 0; w < warp; ++w) pre += s_tot[w];
-            s_base[tid] = pre;
-            // stable scatter, 256 entries per round in their order
-            for (uint32_t i0 = rg.x; i0 < rg.y; i0 += 256) {
-#pragma unroll
-                for (int w = 0; w < kSortWarps; ++w) s_w[w][tid] = 0;
-                __syncthreads();
-                const uint32_t i = i0 + tid;
-                const bool in = i < rg.y;
-                const uint32_t key = DB > 0 && in ? ki[i] : 0u, val = in ? vi[i] : 0u;
-                const uint32_t d = in ? (((by_tri ? val : key) >> shift) & 255u) : 256u;
-                const unsigned peers = __match_any_sync(kFull, d);
-                const uint32_t wrank = __popc(peers & lt);
-                if (in && wrank == 0) s_w[warp][d] = __popc(peers);
-                __syncthreads();
-                {
-                    uint32_t run = s_base[tid];
-#pragma unroll
-                    for (int w = 0; w < kSortWarps; ++w) {
-                        const uint32_t m = s_w[w][tid];
-                        s_w[w][tid] = run;
-                        run += m;
-                    }
-                    s_base[tid] = run;
-                }
-                __syncthreads();
-                if (in) {
-                    const uint32_t pos = rg.x + s_w[warp][d] + wrank;
-                    if (DB > 0) ko[pos] = key;
-                    vo[pos] = val;
-                }
-                __syncthreads();
-            }
-            uint32_t* x = ki;
-            ki = ko;
-            ko = x;
-            x = vi;
-            vi = vo;
-            vo = x;
-        }
-        if (vi != v0)
-            for (uint32_t i = rg.x + tid; i < rg.y; i += 256) {
-                if (DB > 0) k0[i] = ki[i];
-                v0[i] = vi[i];
-            }
-        __syncthreads();
+        if (n > kWarpList && n <= kBlockList) sort_block(s_kv, k0 + rg.x, v0 + rg.x, k0 + rg.x, v0 + rg.x, n, DB > 0);
+    }
+    const uint32_t nc = n_chunks ? *n_chunks : 0u;
+    for (uint32_t i = blockIdx.x; i < nc; i += gridDim.x) {
+        const uint2 ch = chunks[i], rg = ranges[ch.x];
+        const uint32_t lo = rg.x + ch.y * kBlockList;
+        sort_block(s_kv, k0 + lo, v0 + lo, k1 + lo, v1 + lo, (int)min((uint32_t)kBlockList, rg.y - lo), DB > 0);
     }
 }
 
-cudaError_t launch_tile_sort(const ViewTable& vt, const uint2* ranges, int n_tiles, int DB, uint32_t* k0, uint32_t* v0,
-                             uint32_t* k1, uint32_t* v1, cudaStream_t st) {
-    int tri_passes = 1;   // 8-bit digits of the largest triangle index
+// The sorted chunks (k1, v1) of the long lists into one order (k0, v0): an
+// entry's place is its place in its chunk plus the number of smaller entries
+// of every other chunk of the list, found by bisection with that chunk in
+// shared memory.
+__global__ void __launch_bounds__(kSortThreads) k_list_merge(const uint2* __restrict__ ranges, int DB,
+                                                             const uint32_t* __restrict__ n_chunks,
+                                                             const uint2* __restrict__ chunks,
+                                                             const uint32_t* __restrict__ k1,
+                                                             const uint32_t* __restrict__ v1, uint32_t* __restrict__ k0,
+                                                             uint32_t* __restrict__ v0) {
+    __shared__ unsigned long long s_kv[kBlockList];
+    constexpr int E = kBlockList / kSortThreads;
+    const int tid = threadIdx.x;
+    const uint32_t nc = *n_chunks;
+    const auto entry = [&](uint32_t i) { return ((unsigned long long)(DB > 0 ? k1[i] : 0u) << 32) | v1[i]; };
+    for (uint32_t item = blockIdx.x; item < nc; item += gridDim.x) {
+        const uint2 ch = chunks[item], rg = ranges[ch.x];
+        const uint32_t m = (rg.y - rg.x + kBlockList - 1) / kBlockList, lo = rg.x + ch.y * kBlockList;
+        unsigned long long x[E];
+        uint32_t rank[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            rank[e] = tid + e * kSortThreads;
+            x[e] = lo + rank[e] < rg.y ? entry(lo + rank[e]) : ~0ull;
+        }
+        for (uint32_t o = 0; o < m; ++o) {
+            if (o == ch.y) continue;
+            const uint32_t from = rg.x + o * kBlockList;
+            __syncthreads();
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const uint32_t i = tid + e * kSortThreads;
+                s_kv[i] = from + i < rg.y ? entry(from + i) : ~0ull;
+            }
+            __syncthreads();
+            uint32_t pos[E] = {};
+#pragma unroll
+            for (int step = kBlockList / 2; step > 0; step >>= 1)
+#pragma unroll
+                for (int e = 0; e < E; ++e)
+                    if (s_kv[pos[e] + step - 1] < x[e]) pos[e] += step;
+#pragma unroll
+            for (int e = 0; e < E; ++e) rank[e] += pos[e] + (s_kv[pos[e]] < x[e] ? 1u : 0u);
+        }
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if (lo + tid + e * kSortThreads < rg.y) {
+                if (DB > 0) k0[rg.x + rank[e]] = (uint32_t)(x[e] >> 32);
+                v0[rg.x + rank[e]] = (uint32_t)x[e];
+            }
+    }
+}
+
+bool long_lists(const ViewTable& vt) {
     for (int v = 0; v < vt.n; ++v)
-        while (vt.v[v].s_T > 1 << 8 * tri_passes) ++tri_passes;
-    k_tile_sort<<<(n_tiles + kSortWarps - 1) / kSortWarps, 256, 0, st>>>(ranges, n_tiles, DB, tri_passes, k0, v0, k1, v1);
+        if (vt.v[v].s_T > kBlockList) return true;
+    return false;
+}
+
+// CTAs for the chunks of the long lists: as many as full chunks fit the
+// buffers, at most what the device holds at once.
+static int chunk_grid(uint32_t cap) { return persistent_grid((int)(cap / kBlockList) + 1, 2048 / kSortThreads); }
+
+cudaError_t launch_tile_sort(const ViewTable& vt, const uint2* ranges, int n_tiles, int DB, const uint32_t* n_chunks,
+                             const uint2* chunks, uint32_t cap, uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1,
+                             cudaStream_t st) {
+    // Few tiles: fewer of them per CTA, down to one, so that their lists are
+    // sorted side by side (eight always: b 24 -> 50, 256 tiles of 740 entries
+    // 28 -> 53).  Up to four CTAs per SM; two or eight measure alike.
+    int per = 1;
+    while (per < kSortWarps && n_tiles > per * persistent_grid(1 << 30, 4)) per *= 2;
+    const bool lng = long_lists(vt);
+    const int grid = std::max((n_tiles + per - 1) / per, lng ? chunk_grid(cap) : 1);
+    k_tile_sort<<<grid, kSortThreads, 0, st>>>(ranges, n_tiles, per, DB, lng ? n_chunks : nullptr, chunks, k0, v0, k1, v1);
+    note_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_list_merge(const uint2* ranges, int DB, const uint32_t* n_chunks, const uint2* chunks, uint32_t cap,
+                              uint32_t* k0, uint32_t* v0, const uint32_t* k1, const uint32_t* v1, cudaStream_t st) {
+    k_list_merge<<<chunk_grid(cap), kSortThreads, 0, st>>>(ranges, DB, n_chunks, chunks, k1, v1, k0, v0);
     note_launches(1);
     return cudaGetLastError();
 }

@@ -38,6 +38,12 @@ long long launches_total();
 
 constexpr int kEdgeTileW = 32;      // tile width of the edge kernel (its own pixel partition)
 constexpr int kScanBlock = 4096;    // tiles per block of the tile scan (1024 threads x 4)
+// Lists above this length are sorted in chunks of it, by several CTAs.  1,000,000
+// triangles in a 64 x 64 view: 132 us (chunks of 1,024: 174, of 4,096: 148);
+// 200,000 there: 51 (47, 74).
+constexpr int kBlockList = 2048;
+// Chunks that the long lists of `pairs` entries can have.
+constexpr size_t max_chunks(size_t pairs) { return 2 * (pairs / kBlockList) + 1; }
 
 // ---- activation (ds_activate.cu), set-up and binning (ds_bin.cu)
 cudaError_t launch_activate(const SoupDev& s, cudaStream_t st);
@@ -53,19 +59,29 @@ long long view_records(const ViewTable& vt);
 cudaError_t launch_setup(const ViewTable& vt, int n_tiles, SetupRec* recs, uint32_t* tile_count, int4* tbox,
                          uint32_t* zkeys, cudaStream_t st);
 // Scan of the counts: every tile's list range (cut at cap pairs), its cursor
-// for the emission, the number of pairs *total; sets counters[0 ..
-// n_counters-1] to zero.  block_sum: scratch, one word per kScanBlock tiles.
+// for the emission, the number of pairs total[0]; the chunks (tile, index) of
+// the lists above kBlockList entries and their number total[1]; sets
+// counters[0 .. n_counters-1] to zero.  block_sum: scratch, one word per
+// kScanBlock tiles; chunks: max_chunks(cap) items.
 cudaError_t launch_tile_offsets(const uint32_t* count, int n_tiles, uint32_t cap, uint32_t* block_sum, uint2* ranges,
-                                uint32_t* cursor, uint32_t* total, int* counters, int n_counters, cudaStream_t st);
+                                uint32_t* cursor, uint32_t* total, uint2* chunks, int* counters, int n_counters,
+                                cudaStream_t st);
 // Every (tile, triangle) pair into its tile's list: vals the triangles, keys
 // the DB depth bits (not written when DB = 0).  Beyond cap: bit 0 of *status
 // (if status is not NULL).
 cudaError_t launch_emit(const ViewTable& vt, const SetupRec* recs, const int4* tbox, const uint32_t* zkeys, int DB,
                         uint32_t* cursor, uint32_t* keys, uint32_t* vals, uint32_t cap, int* status, cudaStream_t st);
 // Every list by (depth key, triangle), by triangle when DB = 0; k1, v1: scratch
-// of the lists' size.
-cudaError_t launch_tile_sort(const ViewTable& vt, const uint2* ranges, int n_tiles, int DB, uint32_t* k0, uint32_t* v0, uint32_t* k1,
-                             uint32_t* v1, cudaStream_t st);
+// of the lists' size (cap pairs).  Lists above kBlockList entries come out as
+// sorted chunks in (k1, v1), which launch_list_merge brings into order in
+// (k0, v0); n_chunks: total[1] of launch_tile_offsets.  long_lists: whether
+// a list can be that long (a triangle is in a tile's list once).
+bool long_lists(const ViewTable& vt);
+cudaError_t launch_tile_sort(const ViewTable& vt, const uint2* ranges, int n_tiles, int DB, const uint32_t* n_chunks,
+                             const uint2* chunks, uint32_t cap, uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1,
+                             cudaStream_t st);
+cudaError_t launch_list_merge(const uint2* ranges, int DB, const uint32_t* n_chunks, const uint2* chunks, uint32_t cap,
+                              uint32_t* k0, uint32_t* v0, const uint32_t* k1, const uint32_t* v1, cudaStream_t st);
 
 // ---- forward rasteriser (ds_raster.cu)
 // multi: every view reads its own soup (ViewDesc s_*, rec_base) instead of s

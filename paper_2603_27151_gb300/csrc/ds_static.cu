@@ -31,7 +31,8 @@ constexpr size_t kOffKeys0 = align256(kOffZkeys + 4 * kMaxViewTris);
 constexpr size_t kOffVals0 = align256(kOffKeys0 + 4 * kMaxPairs);
 constexpr size_t kOffKeys1 = align256(kOffVals0 + 4 * kMaxPairs);
 constexpr size_t kOffVals1 = align256(kOffKeys1 + 4 * kMaxPairs);
-constexpr size_t kOffCount = align256(kOffVals1 + 4 * kMaxPairs);
+constexpr size_t kOffChunks = align256(kOffVals1 + 4 * kMaxPairs);
+constexpr size_t kOffCount = align256(kOffChunks + sizeof(uint2) * ds::max_chunks(kMaxPairs));
 constexpr size_t kOffCursor = align256(kOffCount + 4 * kMaxTiles);
 constexpr size_t kOffSums = align256(kOffCursor + 4 * kMaxTiles);
 constexpr size_t kOffRanges = align256(kOffSums + 4 * (kMaxTiles / ds::kScanBlock + 1));
@@ -143,6 +144,7 @@ extern "C" DS_API ds_status ds_raster_forward_noalloc(const float* verts, const 
     auto* zkeys = reinterpret_cast<uint32_t*>(base + kOffZkeys);
     uint32_t* keys[2] = {reinterpret_cast<uint32_t*>(base + kOffKeys0), reinterpret_cast<uint32_t*>(base + kOffKeys1)};
     uint32_t* vals[2] = {reinterpret_cast<uint32_t*>(base + kOffVals0), reinterpret_cast<uint32_t*>(base + kOffVals1)};
+    auto* chunks = reinterpret_cast<uint2*>(base + kOffChunks);
     auto* tcount = reinterpret_cast<uint32_t*>(base + kOffCount);
     auto* tcursor = reinterpret_cast<uint32_t*>(base + kOffCursor);
     auto* tsums = reinterpret_cast<uint32_t*>(base + kOffSums);
@@ -165,10 +167,12 @@ extern "C" DS_API ds_status ds_raster_forward_noalloc(const float* verts, const 
     NA_TRY(ds::launch_activate(sd, st));
     ds::set_view_soups(vt, sd);
     NA_TRY(ds::launch_setup(vt, tile_base, recs, tcount, tbox, zkeys, st));
-    NA_TRY(ds::launch_tile_offsets(tcount, tile_base, (uint32_t)kMaxPairs, tsums, ranges, tcursor, dK, counter, 2, st));
-    uint32_t K = 0;   // the one data-dependent size, read back into host stack memory
-    NA_TRY(cudaMemcpyAsync(&K, dK, sizeof(K), cudaMemcpyDeviceToHost, st));
+    NA_TRY(ds::launch_tile_offsets(tcount, tile_base, (uint32_t)kMaxPairs, tsums, ranges, tcursor, dK, chunks, counter, 2, st));
+    // the data-dependent sizes, read back into host stack memory: pairs, chunks of long lists
+    uint32_t sizes[2] = {0, 0};
+    NA_TRY(cudaMemcpyAsync(sizes, dK, sizeof(sizes), cudaMemcpyDeviceToHost, st));
     NA_TRY(cudaStreamSynchronize(st));
+    const uint32_t K = sizes[0];
     if ((long long)K > kMaxPairs)
         return reject(DS_ERR_CAPACITY, "binning produced " + std::to_string(K) +
                                            " (tile, triangle) pairs; the no-alloc limit is 524288");
@@ -176,7 +180,10 @@ extern "C" DS_API ds_status ds_raster_forward_noalloc(const float* verts, const 
     while (tile_bits < 32 && (1ull << tile_bits) < (unsigned long long)tile_base) ++tile_bits;
     const int DB = tile_bits <= 16 ? 16 : 32 - tile_bits;
     NA_TRY(ds::launch_emit(vt, recs, tbox, zkeys, DB, tcursor, keys[0], vals[0], (uint32_t)kMaxPairs, status, st));
-    NA_TRY(ds::launch_tile_sort(vt, ranges, tile_base, DB, keys[0], vals[0], keys[1], vals[1], st));
+    NA_TRY(ds::launch_tile_sort(vt, ranges, tile_base, DB, dK + 1, chunks, (uint32_t)kMaxPairs, keys[0], vals[0], keys[1],
+                                vals[1], st));
+    if (sizes[1] > 0)
+        NA_TRY(ds::launch_list_merge(ranges, DB, dK + 1, chunks, (uint32_t)kMaxPairs, keys[0], vals[0], keys[1], vals[1], st));
     ds::Bg b{};
     for (int i = 0; i < C - 1; ++i) b.c[i] = bg[i];
     const int grid = 0;
