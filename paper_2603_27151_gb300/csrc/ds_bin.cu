@@ -23,8 +23,30 @@ namespace ds {
 
 namespace {
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kOwnTiles = 32;   // boxes of more tiles are shared by the warp
+constexpr int kBinThreads = 256;
+constexpr int kOwnTiles = 32;     // boxes of more tiles are shared by the warp,
+constexpr int kWarpTiles = 1024;  // those of more than this by the CTA
+constexpr int kCtaBoxes = 64;     // as many of them as the CTA's list holds
 }  // namespace
+
+// Records per warp of k_setup and k_emit: 32, or fewer while there are not
+// enough records for eight such warps per SM, so that a few triangles with
+// large boxes are walked by the whole chip (500 full-screen triangles at
+// 1280 x 720: k_setup 394 -> 32 us, k_emit 511 -> 41).  Sixteen warps per SM
+// cost 1.5 us on 16,000 records.
+static int records_per_warp(long long n_records) {
+    int per = 1;
+    while (per < 32 && n_records > (long long)per * persistent_grid(1 << 30, 8)) per *= 2;
+    return per;
+}
+
+// The record of this thread (-1: none).
+__device__ __forceinline__ long long own_record(long long n_records, int per) {
+    const long long warp = blockIdx.x * (long long)(kBinThreads / 32) + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    const long long gid = warp * per + lane;
+    return lane < per && gid < n_records ? gid : -1;
+}
 
 // Upper bound of the biased edge value over the tw x th pixel centres of a
 // tile: a linear function peaks at a corner of the centre grid.
@@ -40,15 +62,29 @@ __device__ __forceinline__ bool tile_may_cover(const SetupRec& r, int tx, int ty
     return true;
 }
 
+// A box that the CTA walks together.
+struct CtaBox {
+    SetupRec r;
+    int4 box;
+    int v, t;
+    uint32_t zkey;
+};
+
 // Calls f(tiles, in, triangle, depth key) for the tiles of the lane's box, four
 // at a time: global tile tiles[k] is one whose pixel centres the triangle may
-// cover if in[k].  All 32 lanes call it (an empty box has z < x).  A lane
-// walks a box of up to kOwnTiles tiles itself; the tiles of a larger one are
-// spread over the warp (a full-screen triangle has thousands, and each costs
-// an atomic's round trip in k_emit; four at a time share one).
+// cover if in[k].  All threads of the CTA call it (an empty box has z < x).  A
+// lane walks a box of a few tiles itself; the tiles of a larger one are spread
+// over the warp, those of a very large one over the CTA (a full-screen triangle
+// has thousands, and each costs an atomic's round trip in k_emit; four at a
+// time share one; 64 of them in a row among 20,000 small ones: k_setup 288 ->
+// 112 us, k_emit 411 -> 169).
 template <class F>
-__device__ __forceinline__ void for_tiles(const ViewTable& vt, int v, const SetupRec& r, int4 box, int t, uint32_t zkey,
-                                          F&& f) {
+__device__ __forceinline__ void for_tiles(const ViewTable& vt, int per, int v, const SetupRec& r, int4 box, int t,
+                                          uint32_t zkey, F&& f) {
+    __shared__ CtaBox s_box[kCtaBoxes];
+    __shared__ int s_n;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
     const int nb = box.z < box.x ? 0 : (box.z - box.x + 1) * (box.w - box.y + 1);
     const auto walk = [&](const SetupRec& q, int vq, int x0, int y0, int bw, int i0, int step, int n, int tq, uint32_t zq) {
         const int tiles_x = vt.v[vq].tiles_x, base = vt.v[vq].tile_base;
@@ -64,8 +100,15 @@ __device__ __forceinline__ void for_tiles(const ViewTable& vt, int v, const Setu
             f(tiles, in, tq, zq);
         }
     };
-    if (nb <= kOwnTiles) walk(r, v, box.x, box.y, box.z - box.x + 1, 0, 1, nb, t, zkey);
-    unsigned wide = __ballot_sync(kFull, nb > kOwnTiles);
+    bool cta = nb > kWarpTiles;
+    if (cta) {
+        const int at = atomicAdd(&s_n, 1);
+        cta = at < kCtaBoxes;
+        if (cta) s_box[at] = CtaBox{r, box, v, t, zkey};
+    }
+    const int own = max(4, kOwnTiles * per / 32);   // fewer records per warp: more lanes idle
+    if (nb <= own) walk(r, v, box.x, box.y, box.z - box.x + 1, 0, 1, nb, t, zkey);
+    unsigned wide = __ballot_sync(kFull, nb > own && !cta);
     while (wide) {
         const int src = __ffs(wide) - 1;
         wide &= wide - 1;
@@ -81,6 +124,12 @@ __device__ __forceinline__ void for_tiles(const ViewTable& vt, int v, const Setu
         const int vs = __shfl_sync(kFull, v, src), ts = __shfl_sync(kFull, t, src);
         walk(q, vs, x0, y0, bw, threadIdx.x & 31, 32, n, ts, __shfl_sync(kFull, zkey, src));
     }
+    __syncthreads();
+    for (int i = 0; i < min(s_n, kCtaBoxes); ++i) {
+        const CtaBox& c = s_box[i];
+        const int bw = c.box.z - c.box.x + 1;
+        walk(c.r, c.v, c.box.x, c.box.y, bw, threadIdx.x, kBinThreads, bw * (c.box.w - c.box.y + 1), c.t, c.zkey);
+    }
 }
 
 // ---------------------------------------------------------------- set-up
@@ -94,19 +143,18 @@ __device__ __forceinline__ int view_of_record(const ViewTable& vt, long long gid
     return v;
 }
 
-// One thread per (view, triangle): project, snap to 1/256 pixel, cull, build
+// One thread per (view, triangle), `per` of them in a warp: project, snap to 1/256 pixel, cull, build
 // the oriented edge functions with the top-left fill rule (Eq. 1 fragments),
 // the perspective factors k_i and the tile rectangle, and count the triangle
 // in every tile whose pixel centres it may cover.
-__global__ void __launch_bounds__(256) k_setup(const __grid_constant__ ViewTable vt, long long n_records,
-                                               SetupRec* __restrict__ recs, uint32_t* __restrict__ tile_count,
-                                               int4* __restrict__ tbox, uint32_t* __restrict__ zkeys) {
-    const long long gid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const bool active = gid < n_records;
+__global__ void __launch_bounds__(kBinThreads) k_setup(const __grid_constant__ ViewTable vt, long long n_records, int per,
+                                                       SetupRec* __restrict__ recs, uint32_t* __restrict__ tile_count,
+                                                       int4* __restrict__ tbox, uint32_t* __restrict__ zkeys) {
+    const long long gid = own_record(n_records, per);
     int v = 0, t = 0;
     SetupRec r;
     int4 box = make_int4(0, 0, -1, -1);
-    if (active) {
+    if (gid >= 0) {
         v = view_of_record(vt, gid);
         t = (int)(gid - vt.v[v].rec_base);
         const DevCam& cam = view_cam(vt, v);
@@ -182,7 +230,7 @@ __global__ void __launch_bounds__(256) k_setup(const __grid_constant__ ViewTable
         tbox[gid] = box;
         zkeys[gid] = zk;
     }
-    for_tiles(vt, v, r, box, t, 0u, [&](const int (&tiles)[4], const bool (&in)[4], int, uint32_t) {
+    for_tiles(vt, per, v, r, box, t, 0u, [&](const int (&tiles)[4], const bool (&in)[4], int, uint32_t) {
 #pragma unroll
         for (int k = 0; k < 4; ++k)
             if (in[k]) atomicAdd(tile_count + tiles[k], 1u);
@@ -218,7 +266,8 @@ cudaError_t launch_setup(const ViewTable& vt, int n_tiles, SetupRec* recs, uint3
     const long long n = view_records(vt);
     cudaError_t e = cudaMemsetAsync(tile_count, 0, sizeof(uint32_t) * (size_t)n_tiles, st);
     if (e != cudaSuccess || n <= 0) return e;
-    k_setup<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(vt, n, recs, tile_count, tbox, zkeys);
+    const int per = records_per_warp(n), cta = per * kBinThreads / 32;
+    k_setup<<<(unsigned)((n + cta - 1) / cta), kBinThreads, 0, st>>>(vt, n, per, recs, tile_count, tbox, zkeys);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -309,14 +358,15 @@ cudaError_t launch_tile_offsets(const uint32_t* count, int n_tiles, uint32_t cap
 // ---------------------------------------------------------------- emission
 // Each pair to the next place of its tile; the key holds the depth bits (none
 // is written without).  Pairs beyond the capacity are dropped and reported.
-__global__ void __launch_bounds__(256) k_emit(const __grid_constant__ ViewTable vt, long long n_records,
-                                              const SetupRec* __restrict__ recs, const int4* __restrict__ tbox,
-                                              const uint32_t* __restrict__ zkeys, int DB, uint32_t* __restrict__ cursor,
-                                              uint32_t* __restrict__ keys, uint32_t* __restrict__ vals, uint32_t cap,
-                                              int* __restrict__ status) {
-    const long long gid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(kBinThreads) k_emit(const __grid_constant__ ViewTable vt, long long n_records, int per,
+                                                      const SetupRec* __restrict__ recs, const int4* __restrict__ tbox,
+                                                      const uint32_t* __restrict__ zkeys, int DB,
+                                                      uint32_t* __restrict__ cursor, uint32_t* __restrict__ keys,
+                                                      uint32_t* __restrict__ vals, uint32_t cap,
+                                                      int* __restrict__ status) {
+    const long long gid = own_record(n_records, per);
     int4 box = make_int4(0, 0, -1, -1);
-    if (gid < n_records) box = tbox[gid];
+    if (gid >= 0) box = tbox[gid];
     int v = 0, t = 0;
     uint32_t zk = 0;
     SetupRec r;
@@ -327,7 +377,7 @@ __global__ void __launch_bounds__(256) k_emit(const __grid_constant__ ViewTable 
         zk = DB > 0 ? (zkeys[gid] & 0x7fffffffu) >> (31 - DB) : 0u;
     }
     bool over = false;
-    for_tiles(vt, v, r, box, t, zk, [&](const int (&tiles)[4], const bool (&in)[4], int tri, uint32_t z) {
+    for_tiles(vt, per, v, r, box, t, zk, [&](const int (&tiles)[4], const bool (&in)[4], int tri, uint32_t z) {
         uint32_t o[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) o[k] = in[k] ? atomicAdd(cursor + tiles[k], 1u) : 0u;
@@ -347,7 +397,9 @@ cudaError_t launch_emit(const ViewTable& vt, const SetupRec* recs, const int4* t
                         uint32_t* cursor, uint32_t* keys, uint32_t* vals, uint32_t cap, int* status, cudaStream_t st) {
     const long long n = view_records(vt);
     if (n <= 0) return cudaSuccess;
-    k_emit<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(vt, n, recs, tbox, zkeys, DB, cursor, keys, vals, cap, status);
+    const int per = records_per_warp(n), cta = per * kBinThreads / 32;
+    k_emit<<<(unsigned)((n + cta - 1) / cta), kBinThreads, 0, st>>>(vt, n, per, recs, tbox, zkeys, DB, cursor, keys, vals,
+                                                                   cap, status);
     note_launches(1);
     return cudaGetLastError();
 }
