@@ -363,8 +363,8 @@ ds_status prepare(ds_ctx* c, int32_t plan_soup, Soup* const* soups, const ds_cam
     DS_TRY(c->tbox.ensure(16 * nvt, "tile boxes"));
     DS_TRY(c->zkeys.ensure(4 * nvt, "depth keys"));
     DS_TRY(c->ranges.ensure(8 * (size_t)n_tiles, "tile ranges"));
-    DS_TRY(c->tcount.ensure(4 * (size_t)n_tiles, "tile counts"));
-    DS_TRY(c->tcursor.ensure(4 * (size_t)n_tiles, "tile cursors"));
+    DS_TRY(c->tcount.ensure(4 * ds::counter_words(n_tiles), "tile counts"));
+    DS_TRY(c->tcursor.ensure(4 * ds::counter_words(n_tiles), "tile cursors"));
     DS_TRY(c->tsums.ensure(4 * ((size_t)n_tiles / ds::kScanBlock + 1), "tile scan sums"));
 
     for (int v = 0; v < vt.n; ++v) {
@@ -398,7 +398,7 @@ ds_status prepare(ds_ctx* c, int32_t plan_soup, Soup* const* soups, const ds_cam
         cudaError_t e = cudaSuccess;
         {
             StageScope p(c, ds::kStEmit, st);
-            e = ds::launch_emit(vt, c->recs.as<ds::SetupRec>(), c->tbox.as<int4>(), c->zkeys.as<uint32_t>(), DB,
+            e = ds::launch_emit(vt, n_tiles, c->recs.as<ds::SetupRec>(), c->tbox.as<int4>(), c->zkeys.as<uint32_t>(), DB,
                                 c->tcursor.as<uint32_t>(), c->keys[0].as<uint32_t>(), c->vals[0].as<uint32_t>(), limit,
                                 status, st);
         }

@@ -40,6 +40,14 @@ static int records_per_warp(long long n_records) {
     return per;
 }
 
+// A CTA's counter of a tile (its count in k_setup, its cursor in k_emit, which
+// have the same records in the same CTAs): tile * step + first.
+struct CounterAt {
+    int step, first;
+    __device__ explicit CounterAt(bool split)
+        : step(split ? kSplitWays * kSplitWords : 1), first(split ? (int)(blockIdx.x % kSplitWays) * kSplitWords : 0) {}
+};
+
 // The record of this thread (-1: none).
 __device__ __forceinline__ long long own_record(long long n_records, int per) {
     const long long warp = blockIdx.x * (long long)(kBinThreads / 32) + (threadIdx.x >> 5);
@@ -148,9 +156,10 @@ __device__ __forceinline__ int view_of_record(const ViewTable& vt, long long gid
 // the perspective factors k_i and the tile rectangle, and count the triangle
 // in every tile whose pixel centres it may cover.
 __global__ void __launch_bounds__(kBinThreads) k_setup(const __grid_constant__ ViewTable vt, long long n_records, int per,
-                                                       SetupRec* __restrict__ recs, uint32_t* __restrict__ tile_count,
+                                                       bool split, SetupRec* __restrict__ recs, uint32_t* __restrict__ tile_count,
                                                        int4* __restrict__ tbox, uint32_t* __restrict__ zkeys) {
     const long long gid = own_record(n_records, per);
+    const CounterAt at(split);
     int v = 0, t = 0;
     SetupRec r;
     int4 box = make_int4(0, 0, -1, -1);
@@ -233,7 +242,7 @@ __global__ void __launch_bounds__(kBinThreads) k_setup(const __grid_constant__ V
     for_tiles(vt, per, v, r, box, t, 0u, [&](const int (&tiles)[4], const bool (&in)[4], int, uint32_t) {
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-            if (in[k]) atomicAdd(tile_count + tiles[k], 1u);
+            if (in[k]) atomicAdd(tile_count + tiles[k] * at.step + at.first, 1u);
     });
 }
 
@@ -264,10 +273,11 @@ void set_view_soups(ViewTable& vt, const SoupDev& s) {
 cudaError_t launch_setup(const ViewTable& vt, int n_tiles, SetupRec* recs, uint32_t* tile_count, int4* tbox,
                          uint32_t* zkeys, cudaStream_t st) {
     const long long n = view_records(vt);
-    cudaError_t e = cudaMemsetAsync(tile_count, 0, sizeof(uint32_t) * (size_t)n_tiles, st);
+    cudaError_t e = cudaMemsetAsync(tile_count, 0, sizeof(uint32_t) * counter_words(n_tiles), st);
     if (e != cudaSuccess || n <= 0) return e;
     const int per = records_per_warp(n), cta = per * kBinThreads / 32;
-    k_setup<<<(unsigned)((n + cta - 1) / cta), kBinThreads, 0, st>>>(vt, n, per, recs, tile_count, tbox, zkeys);
+    k_setup<<<(unsigned)((n + cta - 1) / cta), kBinThreads, 0, st>>>(vt, n, per, split_counters(n_tiles), recs, tile_count, tbox,
+                                                                    zkeys);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -294,23 +304,28 @@ __global__ void __launch_bounds__(1024) k_tile_sums(const uint32_t* __restrict__
 // Exclusive scan of the tile counts: every tile's range in the lists (cut at
 // the capacity `cap`) and its cursor for k_emit, the number of pairs total[0],
 // the chunks of the lists above kBlockList entries and their number total[1],
-// and the tile kernels' work counters set to zero.  Block b adds up the sums of
-// the blocks before it itself (at most 4,096 for the largest call).
+// and the tile kernels' work counters set to zero.  A thread has four tiles,
+// or the four counters of one (kSplit).  Block b adds up the sums of the
+// blocks before it itself (at most 4,096 for the largest call).
+template <bool kSplit>
 __global__ void __launch_bounds__(1024) k_tile_offsets(const uint32_t* __restrict__ count, int n, uint32_t cap,
                                                        const uint32_t* __restrict__ block_sum, uint2* __restrict__ ranges,
                                                        uint32_t* __restrict__ cursor, uint32_t* __restrict__ total,
                                                        uint2* __restrict__ chunks, int* __restrict__ counters,
                                                        int n_counters) {
     __shared__ uint32_t wsum[32], wpre[32];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, base = blockIdx.x * kScanBlock + 4 * tid;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int base = kSplit ? tid : blockIdx.x * kScanBlock + 4 * tid;
+    constexpr int kTiles = kSplit ? 1 : 4;   // tiles of a thread
     if (gridDim.x == 1 && tid == 0) total[1] = 0;   // else k_tile_sums has cleared it
     uint32_t before = 0;
     for (int b = tid; b < (int)blockIdx.x; b += 1024) before += block_sum[b];
     before = __reduce_add_sync(kFull, before);
+    const auto slot = [&](int k) { return kSplit ? (base * kSplitWays + k) * kSplitWords : base + k; };
     uint32_t x[4], sum = 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        x[k] = base + k < n ? count[base + k] : 0u;
+        x[k] = base + (kSplit ? 0 : k) < n ? count[slot(k)] : 0u;
         sum += x[k];
     }
     uint32_t inc = sum;
@@ -325,18 +340,21 @@ __global__ void __launch_bounds__(1024) k_tile_offsets(const uint32_t* __restric
     uint32_t off = inc - sum;
     for (int w = 0; w < 32; ++w) off += wpre[w] + (w < warp ? wsum[w] : 0u);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        if (base + k < n) {
-            const uint32_t lo = min(off, cap), hi = min(off + x[k], cap);
-            ranges[base + k] = make_uint2(lo, hi);
-            cursor[base + k] = off;
-            if (hi - lo > kBlockList) {
-                const uint32_t m = (hi - lo + kBlockList - 1) / kBlockList, at = atomicAdd(total + 1, m);
-                for (uint32_t c = 0; c < m; ++c) chunks[at + c] = make_uint2((uint32_t)(base + k), c);
-            }
-            if (base + k == n - 1) *total = off + x[k];
+    for (int t = 0; t < kTiles; ++t) {
+        const uint32_t first = off;
+        if (base + t >= n) break;
+#pragma unroll
+        for (int k = t * (4 / kTiles); k < (t + 1) * (4 / kTiles); ++k) {
+            cursor[slot(k)] = off;
+            off += x[k];
         }
-        off += x[k];
+        const uint32_t lo = min(first, cap), hi = min(off, cap);
+        ranges[base + t] = make_uint2(lo, hi);
+        if (hi - lo > kBlockList) {
+            const uint32_t m = (hi - lo + kBlockList - 1) / kBlockList, at = atomicAdd(total + 1, m);
+            for (uint32_t c = 0; c < m; ++c) chunks[at + c] = make_uint2((uint32_t)(base + t), c);
+        }
+        if (base + t == n - 1) *total = off;
     }
     if (blockIdx.x == 0 && tid < n_counters) counters[tid] = 0;
 }
@@ -349,8 +367,8 @@ cudaError_t launch_tile_offsets(const uint32_t* count, int n_tiles, uint32_t cap
         k_tile_sums<<<nblk, 1024, 0, st>>>(count, n_tiles, block_sum, total);
         note_launches(1);
     }
-    k_tile_offsets<<<nblk, 1024, 0, st>>>(count, n_tiles, cap, block_sum, ranges, cursor, total, chunks, counters,
-                                             n_counters);
+    const auto kernel = split_counters(n_tiles) ? k_tile_offsets<true> : k_tile_offsets<false>;
+    kernel<<<nblk, 1024, 0, st>>>(count, n_tiles, cap, block_sum, ranges, cursor, total, chunks, counters, n_counters);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -358,13 +376,14 @@ cudaError_t launch_tile_offsets(const uint32_t* count, int n_tiles, uint32_t cap
 // ---------------------------------------------------------------- emission
 // Each pair to the next place of its tile; the key holds the depth bits (none
 // is written without).  Pairs beyond the capacity are dropped and reported.
-__global__ void __launch_bounds__(kBinThreads) k_emit(const __grid_constant__ ViewTable vt, long long n_records, int per,
+__global__ void __launch_bounds__(kBinThreads) k_emit(const __grid_constant__ ViewTable vt, long long n_records, int per, bool split,
                                                       const SetupRec* __restrict__ recs, const int4* __restrict__ tbox,
                                                       const uint32_t* __restrict__ zkeys, int DB,
                                                       uint32_t* __restrict__ cursor, uint32_t* __restrict__ keys,
                                                       uint32_t* __restrict__ vals, uint32_t cap,
                                                       int* __restrict__ status) {
     const long long gid = own_record(n_records, per);
+    const CounterAt at(split);
     int4 box = make_int4(0, 0, -1, -1);
     if (gid >= 0) box = tbox[gid];
     int v = 0, t = 0;
@@ -380,7 +399,7 @@ __global__ void __launch_bounds__(kBinThreads) k_emit(const __grid_constant__ Vi
     for_tiles(vt, per, v, r, box, t, zk, [&](const int (&tiles)[4], const bool (&in)[4], int tri, uint32_t z) {
         uint32_t o[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) o[k] = in[k] ? atomicAdd(cursor + tiles[k], 1u) : 0u;
+        for (int k = 0; k < 4; ++k) o[k] = in[k] ? atomicAdd(cursor + tiles[k] * at.step + at.first, 1u) : 0u;
 #pragma unroll
         for (int k = 0; k < 4; ++k)
             if (in[k] && o[k] < cap) {
@@ -393,13 +412,13 @@ __global__ void __launch_bounds__(kBinThreads) k_emit(const __grid_constant__ Vi
     if (over && status) atomicOr(status, 1);
 }
 
-cudaError_t launch_emit(const ViewTable& vt, const SetupRec* recs, const int4* tbox, const uint32_t* zkeys, int DB,
+cudaError_t launch_emit(const ViewTable& vt, int n_tiles, const SetupRec* recs, const int4* tbox, const uint32_t* zkeys, int DB,
                         uint32_t* cursor, uint32_t* keys, uint32_t* vals, uint32_t cap, int* status, cudaStream_t st) {
     const long long n = view_records(vt);
     if (n <= 0) return cudaSuccess;
     const int per = records_per_warp(n), cta = per * kBinThreads / 32;
-    k_emit<<<(unsigned)((n + cta - 1) / cta), kBinThreads, 0, st>>>(vt, n, per, recs, tbox, zkeys, DB, cursor, keys, vals,
-                                                                   cap, status);
+    k_emit<<<(unsigned)((n + cta - 1) / cta), kBinThreads, 0, st>>>(vt, n, per, split_counters(n_tiles), recs, tbox, zkeys, DB,
+                                                                   cursor, keys, vals, cap, status);
     note_launches(1);
     return cudaGetLastError();
 }

@@ -53,6 +53,19 @@ cudaError_t launch_activate(const SoupDev& s, cudaStream_t st);
 void set_view_soups(ViewTable& vt, const SoupDev& s);
 void set_view_soups(ViewTable& vt, const SoupDev* const* soups);
 long long view_records(const ViewTable& vt);
+// Few tiles have four counters (counts and cursors) each, in memory lines of
+// their own: atomics on one address, or on one line, are served one after the
+// other.  k_setup and k_emit on 200,000 triangles in a 256 x 256 view: 55 and
+// 37 us with one word per tile, 17 and 14 now; in a 64 x 64 view 53 and 52,
+// 28 and 22 (lines of their own alone: 55 and 55; half lines: 33 and 32).
+// With more tiles the pairs spread by themselves (1,920 tiles: 13 and 14
+// either way).
+constexpr int kSplitTiles = 1024, kSplitWays = 4, kSplitWords = 32;
+static_assert(kSplitTiles * kSplitWays <= kScanBlock, "one block scans split counters");
+constexpr bool split_counters(int n_tiles) { return n_tiles <= kSplitTiles; }
+constexpr size_t counter_words(int n_tiles) {
+    return split_counters(n_tiles) ? (size_t)n_tiles * kSplitWays * kSplitWords : (size_t)n_tiles;
+}
 // One set-up record (and tile box, depth key) per (view, triangle of the
 // view's soup), at rec_base + triangle; tile_count [n_tiles]: the triangles
 // of every tile.
@@ -69,7 +82,7 @@ cudaError_t launch_tile_offsets(const uint32_t* count, int n_tiles, uint32_t cap
 // Every (tile, triangle) pair into its tile's list: vals the triangles, keys
 // the DB depth bits (not written when DB = 0).  Beyond cap: bit 0 of *status
 // (if status is not NULL).
-cudaError_t launch_emit(const ViewTable& vt, const SetupRec* recs, const int4* tbox, const uint32_t* zkeys, int DB,
+cudaError_t launch_emit(const ViewTable& vt, int n_tiles, const SetupRec* recs, const int4* tbox, const uint32_t* zkeys, int DB,
                         uint32_t* cursor, uint32_t* keys, uint32_t* vals, uint32_t cap, int* status, cudaStream_t st);
 // Every list by (depth key, triangle), by triangle when DB = 0; k1, v1: scratch
 // of the lists' size (cap pairs).  Lists above kBlockList entries come out as

@@ -4,6 +4,7 @@
 // counters) lives in one file-scope device array of fixed size; the caller
 // passes inputs and outputs as usual.  No cudaMalloc, cudaFree or other
 // allocating call is made.
+#include <algorithm>
 #include <cstring>
 #include <mutex>
 #include <string>
@@ -33,8 +34,9 @@ constexpr size_t kOffKeys1 = align256(kOffVals0 + 4 * kMaxPairs);
 constexpr size_t kOffVals1 = align256(kOffKeys1 + 4 * kMaxPairs);
 constexpr size_t kOffChunks = align256(kOffVals1 + 4 * kMaxPairs);
 constexpr size_t kOffCount = align256(kOffChunks + sizeof(uint2) * ds::max_chunks(kMaxPairs));
-constexpr size_t kOffCursor = align256(kOffCount + 4 * kMaxTiles);
-constexpr size_t kOffSums = align256(kOffCursor + 4 * kMaxTiles);
+constexpr size_t kCounters = std::max(ds::counter_words(ds::kSplitTiles), (size_t)kMaxTiles);
+constexpr size_t kOffCursor = align256(kOffCount + 4 * kCounters);
+constexpr size_t kOffSums = align256(kOffCursor + 4 * kCounters);
 constexpr size_t kOffRanges = align256(kOffSums + 4 * (kMaxTiles / ds::kScanBlock + 1));
 constexpr size_t kOffMisc = align256(kOffRanges + 8 * kMaxTiles);
 constexpr size_t kStaticBytes = align256(kOffMisc + 256);   // about 21 MiB
@@ -179,7 +181,7 @@ extern "C" DS_API ds_status ds_raster_forward_noalloc(const float* verts, const 
     int tile_bits = 0;
     while (tile_bits < 32 && (1ull << tile_bits) < (unsigned long long)tile_base) ++tile_bits;
     const int DB = tile_bits <= 16 ? 16 : 32 - tile_bits;
-    NA_TRY(ds::launch_emit(vt, recs, tbox, zkeys, DB, tcursor, keys[0], vals[0], (uint32_t)kMaxPairs, status, st));
+    NA_TRY(ds::launch_emit(vt, tile_base, recs, tbox, zkeys, DB, tcursor, keys[0], vals[0], (uint32_t)kMaxPairs, status, st));
     NA_TRY(ds::launch_tile_sort(vt, ranges, tile_base, DB, dK + 1, chunks, (uint32_t)kMaxPairs, keys[0], vals[0], keys[1],
                                 vals[1], st));
     if (sizes[1] > 0)
