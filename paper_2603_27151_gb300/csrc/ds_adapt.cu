@@ -128,6 +128,55 @@ struct RebuildTap {
 constexpr unsigned kOneTexel = 0xfffffc00u;
 constexpr int kRebuildItems = 2;   // items in flight per thread
 
+// The source of vertex v of the children with split code op > 0.
+__device__ __forceinline__ RebuildTap rebuild_tap(int N, int op, int v) {
+    int i, j;
+    texel_ij(N, v, i, j);
+    int P[3][3];
+    child_corners(op, P);
+    const int X = (N - i - j) * P[0][1] + i * P[1][1] + j * P[2][1];
+    const int Y = (N - i - j) * P[0][2] + i * P[1][2] + j * P[2][2];
+    if ((X & 1) == 0 && (Y & 1) == 0)
+        return RebuildTap{kOneTexel | (unsigned)texel_index(N, X >> 1, Y >> 1), 0.f, 0.f};
+    const Cell cl = find_cell(N, __fdiv_rn((float)X, (float)(2 * N)), __fdiv_rn((float)Y, (float)(2 * N)));
+    return RebuildTap{(unsigned)(cl.k0 | (cl.k1 << 10) | (cl.k2 << 20)), cl.wa, cl.wb};
+}
+
+__device__ __forceinline__ float rebuild_mix(float a, float b, float d, const RebuildTap& tp) {
+    return interp(a, b, d, tp.wa, tp.wb);
+}
+__device__ __forceinline__ float4 rebuild_mix(float4 a, float4 b, float4 d, const RebuildTap& tp) {
+    return make_float4(interp(a.x, b.x, d.x, tp.wa, tp.wb), interp(a.y, b.y, d.y, tp.wa, tp.wb),
+                       interp(a.z, b.z, d.z, tp.wa, tp.wb), interp(a.w, b.w, d.w, tp.wa, tp.wb));
+}
+
+// One level of few triangles, or of channels that the table below does not
+// suit: a thread per texel, which finds the source itself and goes through the
+// channels.  Bound by latency (level 5 of 50 triangles: 34 us for the whole
+// call, 43 with a table in every CTA).
+template <bool kVec>
+__global__ void __launch_bounds__(256) k_rebuild_texels(const float* __restrict__ gin, int N, int C,
+                                                        const int* __restrict__ plan, int n_out,
+                                                        float* __restrict__ gout) {
+    using Item = std::conditional_t<kVec, float4, float>;
+    const int V = (N + 1) * (N + 2) / 2, per = kVec ? C / 4 : C;
+    const long long n = (long long)n_out * V, step = (long long)gridDim.x * blockDim.x;
+    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += step) {
+        const int k = (int)(q / V), v = (int)(q - (long long)k * V);
+        const int code = __ldg(plan + k), op = code & 7;
+        const RebuildTap tp = op > 0 ? rebuild_tap(N, op, v) : RebuildTap{kOneTexel | (unsigned)v, 0.f, 0.f};
+        const Item* g = reinterpret_cast<const Item*>(gin) + (size_t)(code >> 3) * (unsigned)(V * per);
+        Item* d = reinterpret_cast<Item*>(gout) + (size_t)q * per;
+        const Item* a = g + (tp.k & 1023u) * per;
+        if (tp.k < kOneTexel) {
+            const Item *b = g + ((tp.k >> 10) & 1023u) * per, *e = g + ((tp.k >> 20) & 1023u) * per;
+            for (int c = 0; c < per; ++c) d[c] = rebuild_mix(__ldg(a + c), __ldg(b + c), __ldg(e + c), tp);
+        } else {
+            for (int c = 0; c < per; ++c) d[c] = __ldg(a + c);
+        }
+    }
+}
+
 // One level.  The source of a child's texel depends on its code and vertex
 // only: every CTA tabulates the six splits first (shared memory), then the
 // items, V texels of C / 4 channel groups per triangle (scalar channels when
@@ -145,18 +194,7 @@ __global__ void __launch_bounds__(256, 5) k_rebuild_level(const float* __restric
     const int V = (N + 1) * (N + 2) / 2;
     for (int q = threadIdx.x; q < 6 * V; q += blockDim.x) {
         const int op = q / V + 1, v = q - (op - 1) * V;
-        int i, j;
-        texel_ij(N, v, i, j);
-        int P[3][3];
-        child_corners(op, P);
-        const int X = (N - i - j) * P[0][1] + i * P[1][1] + j * P[2][1];
-        const int Y = (N - i - j) * P[0][2] + i * P[1][2] + j * P[2][2];
-        if ((X & 1) == 0 && (Y & 1) == 0) {
-            taps[q] = RebuildTap{kOneTexel | (unsigned)texel_index(N, X >> 1, Y >> 1), 0.f, 0.f};
-        } else {
-            const Cell cl = find_cell(N, __fdiv_rn((float)X, (float)(2 * N)), __fdiv_rn((float)Y, (float)(2 * N)));
-            taps[q] = RebuildTap{(unsigned)(cl.k0 | (cl.k1 << 10) | (cl.k2 << 20)), cl.wa, cl.wb};
-        }
+        taps[q] = rebuild_tap(N, op, v);
     }
     __syncthreads();
     // items: channel group c of texel r of output triangle k; a thread keeps
@@ -198,15 +236,7 @@ __global__ void __launch_bounds__(256, 5) k_rebuild_level(const float* __restric
 #pragma unroll
         for (int u = 0; u < kRebuildItems; ++u) {
             if (u >= n) break;
-            if (tp[u].k < kOneTexel) {
-                if constexpr (kVec)
-                    a[u] = make_float4(interp(a[u].x, b[u].x, d[u].x, tp[u].wa, tp[u].wb),
-                                       interp(a[u].y, b[u].y, d[u].y, tp[u].wa, tp[u].wb),
-                                       interp(a[u].z, b[u].z, d[u].z, tp[u].wa, tp[u].wb),
-                                       interp(a[u].w, b[u].w, d[u].w, tp[u].wa, tp[u].wb));
-                else
-                    a[u] = interp(a[u], b[u], d[u], tp[u].wa, tp[u].wb);
-            }
+            if (tp[u].k < kOneTexel) a[u] = rebuild_mix(a[u], b[u], d[u], tp[u]);
             __stcs(out + dst[u], a[u]);
         }
     }
@@ -287,19 +317,35 @@ cudaError_t launch_rebuild(const float* verts, const float* tex, int T, const in
         const float* in = tex + off_in;
         float* out = tex_out + off_out;
         const bool vec = C % 4 == 0 && (((uintptr_t)in | (uintptr_t)out) & 15) == 0;
-        const size_t smem = sizeof(RebuildTap) * 6 * (size_t)V;
-        const auto run = [&](auto kernel) {
-            cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            const int per = vec ? C / 4 : C;
-            const long long items = (long long)n_out * V * per;
-            // at least eight items per thread; a multiple of `per` CTAs
-            long long grid = std::min<long long>((items + 2047) / 2048, persistent_grid(1 << 30, 5));
-            grid = (grid + per - 1) / per * per;
-            kernel<<<(unsigned)grid, 256, smem, st>>>(in, N, C, plan_dev, n_out, out);
-            return cudaGetLastError();
-        };
-        const cudaError_t e = vec ? run(k_rebuild_level<true>) : run(k_rebuild_level<false>);
+        // The table pays when a CTA has many more texels than it tabulates, and
+        // only where a texel's items are a power of two (level 5, table / texels:
+        // C = 8, 2,000 triangles 65 / 53 us, 8,000 110 / 113, 32,000 273 / 331;
+        // C = 16, 1,000 64 / 56, 4,000 103 / 117; C = 12, 32,000 580 / 419).
+        // Scalar channels: C = 2, 8,000 92 / 84, 16,000 126 / 136; C = 6, 32,000
+        // 819 / 360.
+        const int per = vec ? C / 4 : C;
+        const bool table = (per & (per - 1)) == 0 && (vec ? (long long)n_out * per >= 6000 : per <= 2 && n_out >= 16000);
+        cudaError_t e = cudaSuccess;
+        if (!table) {
+            const long long texels = (long long)n_out * V;
+            const int grid = persistent_grid((int)std::min<long long>((texels + 255) / 256, 1 << 30), 16);
+            if (vec) k_rebuild_texels<true><<<grid, 256, 0, st>>>(in, N, C, plan_dev, n_out, out);
+            else k_rebuild_texels<false><<<grid, 256, 0, st>>>(in, N, C, plan_dev, n_out, out);
+            e = cudaGetLastError();
+        } else {
+            const size_t smem = sizeof(RebuildTap) * 6 * (size_t)V;
+            const auto run = [&](auto kernel) {
+                cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                if (e != cudaSuccess) return e;
+                const long long items = (long long)n_out * V * per;
+                // at least eight items per thread; a multiple of `per` CTAs
+                long long grid = std::min<long long>((items + 2047) / 2048, persistent_grid(1 << 30, 5));
+                grid = (grid + per - 1) / per * per;
+                kernel<<<(unsigned)grid, 256, smem, st>>>(in, N, C, plan_dev, n_out, out);
+                return cudaGetLastError();
+            };
+            e = vec ? run(k_rebuild_level<true>) : run(k_rebuild_level<false>);
+        }
         if (e != cudaSuccess) return e;
         note_launches(1);
         off_in += (size_t)T * V * C;
