@@ -377,9 +377,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_loss_l1_ssim(const __grid_const
 }
 
 // ---------------------------------------------------------------- small calls
-// Calls of at most one wave of 64 x 16 tiles (two CTAs per SM): one CTA per
-// tile, the whole halo blurred on its own.  More arithmetic per pixel than the
-// march, but no chain of steps (4 views of 256 x 200: 34 against 40 us).
+// Calls of few tiles, and images whose strips or segments are mostly empty: one
+// CTA per 64 x 16 tile, the whole halo blurred on its own.  More arithmetic per
+// pixel than the march, but no chain of steps (4 views of 256 x 200: 34 against
+// 40 us), and less of it past the image's edges (64 images of 512 x 16: 56
+// against 101).
 constexpr int kTileX = 64, kTileY = 16;
 constexpr int kTileIX = kTileX + 4 * kR, kTileIY = kTileY + 4 * kR;   // staged input 84 x 36
 constexpr int kTileMX = kTileX + 2 * kR, kTileMY = kTileY + 2 * kR;   // moment region 74 x 26
@@ -673,7 +675,15 @@ cudaError_t launch_loss_l1_ssim(int n_views, int S, int Co, const int* hw, const
     };
     long long n_tiles = 0;
     for (int v = 0; v < n_views; ++v) n_tiles += S * tiles(hw[2 * v], hw[2 * v + 1]);
-    const bool small = n_tiles <= 2 * sms;
+    // The tile kernel's cost in the same unit, a step of the march (about 12 us
+    // with three channels): two CTAs fill an SM for 2.3 steps, and what is
+    // left over after whole waves takes 1.6 or, above one CTA per SM, 2.6.
+    // Over 236 shapes from 1 to 1,920 columns, 16 to 1,080 rows and 1 to 64
+    // images the slower kernel is picked once, by 0.6%; with the tile kernel
+    // up to one wave and the march above it was up to 79% (64 images of
+    // 512 x 16).
+    const long long left = n_tiles % (2 * sms);
+    const bool small = 2.3 * (double)(n_tiles / (2 * sms)) + (left == 0 ? 0.0 : left <= sms ? 1.6 : 2.6) <= best;
     t->rows = kStep * steps - 4 * kR;
     long long cta = 0;
     for (int v = 0; v < n_views; ++v) {
