@@ -571,9 +571,10 @@ DS_API ds_status ds_set_tuning(ds_ctx* ctx, const ds_tuning* t);
 DS_API ds_status ds_get_tuning(ds_ctx* ctx, ds_tuning* t);
 
 /* Autotune the context's tuning on one workload: coordinate search over tile
- * shape {8x32, 16x16, 32x8}, depth bits {16, 8, 0}, chunk {64, 128, 256} and
- * CTAs per SM {occupancy, 2, 3}, each candidate timed (median of `reps` in
- * [1, 100] after one untimed run) with CUDA events on `stream` over
+ * shape {8x32, 16x16, 32x8}, depth bits {16, 8, 0}, chunk {64, 128, 256} (where
+ * the timed calls use it) and CTAs per SM {occupancy, 2, 3}, each candidate
+ * timed (median of `reps` in [1, 100] after one untimed run) with CUDA events
+ * on `stream` over
  * ds_raster_forward (mode) and, when gin is non-NULL, ds_raster_backward with
  * DS_G_ALL | DS_OVERWRITE into grad_verts / grad_tex; or, when lv is
  * non-NULL, over ds_raster_train_l2 with those loss views and scale.

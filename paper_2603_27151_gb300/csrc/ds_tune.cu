@@ -94,7 +94,12 @@ extern "C" ds_status ds_autotune(ds_ctx* c, int32_t soup_id, const ds_camera* ca
     const int dbits[] = {-1, 8, 0};
     const int chunks[] = {64, 128, 256};
     const int blocks[] = {0, 2, 3};
+    // forwards of one and two samples stage 32 triangles per warp whatever the
+    // chunk: alone (no backward, loss or fragment counts) they leave it as it is
+    bool uses_chunk = lv || gin || S > 2;
+    for (int v = 0; out && v < n_views; ++v) uses_chunk = uses_chunk || out[v].n_front;
     for (int knob = 0; knob < 4; ++knob) {
+        if (knob == 2 && !uses_chunk) continue;
         const int* vals = knob == 0 ? tiles : knob == 1 ? dbits : knob == 2 ? chunks : blocks;
         for (int i = 0; i < 3; ++i) {
             ds_tuning t = cur;
