@@ -648,8 +648,9 @@ DS_API ds_status ds_server_destroy(ds_server* srv);
 
 /* Profiling (off by default; no paper counterpart: instrumentation).  While
  * enabled, every pipeline stage that a call on this context launches
- * (activate, setup, scan, emit, sort, raster_fwd, count, geom,
- * raster_bwd, edge_bwd, finish) is bracketed by two CUDA events recorded on the caller's stream.
+ * (activate, setup, scan, emit, sort, ranges -- written by the scan, no
+ * launch of its own --, raster_fwd, count, geom, raster_bwd, edge_bwd,
+ * finish, train) is bracketed by two CUDA events recorded on the caller's stream.
  * ds_profile_read waits for those events and returns, for stage index
  * `stage` in [0, ds_profile_stages()), its name (static host string), the
  * number of times it ran and its summed device time in ms since the last

@@ -11,9 +11,11 @@
 
 namespace ds {
 
-// Pipeline stages timed by the optional profiler (ds_profile_*).
+// Pipeline stages timed by the optional profiler (ds_profile_*).  The scan
+// writes the tile ranges, too: kStRanges has no launch and keeps its name and
+// the indices of the stages behind it.
 enum Stage {
-    kStActivate, kStSetup, kStScan, kStEmit, kStSort,
+    kStActivate, kStSetup, kStScan, kStEmit, kStSort, kStRanges,
     kStRasterFwd, kStCount, kStGeom, kStRasterBwd, kStEdgeBwd, kStFinish, kStTrain, kNumStages
 };
 extern const char* const kStageNames[kNumStages];

@@ -335,7 +335,7 @@ cudaError_t launch_raster_count(const ViewTable& vt, const SoupDev& s, const Set
     return cudaGetLastError();
 }
 
-const char* const kStageNames[kNumStages] = {"activate", "setup", "scan", "emit", "sort",
+const char* const kStageNames[kNumStages] = {"activate", "setup", "scan", "emit", "sort", "ranges",
                                              "raster_fwd", "count", "geom", "raster_bwd", "edge_bwd",
                                              "finish", "train"};
 
