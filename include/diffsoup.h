@@ -554,9 +554,8 @@ DS_API ds_status ds_ctx_status(ds_ctx* ctx);
  * decomposition of Eq. 5 and Algorithm A1; every setting computes the same
  * result).  tile_w: tile width in pixels, 8, 16 or 32 (tiles hold 256 pixels,
  * so 8x32, 16x16 or 32x8).  depth_bits: bits of quantised nearest depth in
- * the bin key that order each tile's list front to back for the early exit,
- * -1 = 16 (or fewer when the tile index needs the bits), 0 = none (lists in
- * the order of the triangles).
+ * the key that orders each tile's list front to back for the early exit, -1 =
+ * 16, 0 = none (lists in the order of the triangles).
  * blocks_per_sm: CTAs per SM of the persistent tile kernels, 0 = each
  * kernel's occupancy limit.  chunk: triangles staged in shared memory per
  * round, a multiple of 32 in [32, 256] (forwards of one and two samples stage

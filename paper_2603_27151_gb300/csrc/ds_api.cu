@@ -224,12 +224,6 @@ ds_status prof_flush(ds_ctx* c) {
     return DS_OK;
 }
 
-int bits_for(uint32_t n_values) {   // bits needed for indices 0 .. n_values-1
-    int b = 0;
-    while (b < 32 && (1ull << b) < n_values) ++b;
-    return b;
-}
-
 ds::SoupDev soup_dev(const Soup& s) {
     ds::SoupDev d;
     d.verts = s.verts;
@@ -386,8 +380,7 @@ ds_status prepare(ds_ctx* c, int32_t plan_soup, Soup* const* soups, const ds_cam
     }
     uint32_t cap = pair_capacity(c);
     const bool wait = sync || cap == 0;
-    const int tile_bits = bits_for((uint32_t)n_tiles);
-    const int DB = std::min(c->tune.depth_bits >= 0 ? c->tune.depth_bits : 16, 32 - tile_bits);
+    const int DB = c->tune.depth_bits >= 0 ? c->tune.depth_bits : 16;
     auto offsets = [&](uint32_t limit) {
         StageScope p(c, ds::kStScan, st);
         return ds::launch_tile_offsets(c->tcount.as<uint32_t>(), n_tiles, limit, c->tsums.as<uint32_t>(),

@@ -178,9 +178,7 @@ extern "C" DS_API ds_status ds_raster_forward_noalloc(const float* verts, const 
     if ((long long)K > kMaxPairs)
         return reject(DS_ERR_CAPACITY, "binning produced " + std::to_string(K) +
                                            " (tile, triangle) pairs; the no-alloc limit is 524288");
-    int tile_bits = 0;
-    while (tile_bits < 32 && (1ull << tile_bits) < (unsigned long long)tile_base) ++tile_bits;
-    const int DB = tile_bits <= 16 ? 16 : 32 - tile_bits;
+    const int DB = 16;
     NA_TRY(ds::launch_emit(vt, tile_base, recs, tbox, zkeys, DB, tcursor, keys[0], vals[0], (uint32_t)kMaxPairs, status, st));
     NA_TRY(ds::launch_tile_sort(vt, ranges, tile_base, DB, dK + 1, chunks, (uint32_t)kMaxPairs, keys[0], vals[0], keys[1],
                                 vals[1], st));

@@ -87,13 +87,12 @@ __device__ __forceinline__ WorkItem decode_item(const ViewTable& vt, int item) {
 }
 
 // Upper bound on the inverse depth of every triangle whose sort key is at
-// least `key`: the key's depth bits are the top DB bits of the nearest
-// vertex depth, so the float they encode is <= that depth.  The bound is
-// widened by 2^-10 to cover the rounding of rho (a few ulps).
+// least `key`: the key is the top DB bits of the nearest vertex depth, so the
+// float they encode is <= that depth.  The bound is widened by 2^-10 to cover
+// the rounding of rho (a few ulps).
 __device__ __forceinline__ float rho_bound(uint32_t key, int DB) {
     if (DB <= 0) return __int_as_float(0x7f800000);
-    const uint32_t q = key & ((1u << DB) - 1u);
-    const float zq = __uint_as_float(q << (31 - DB));
+    const float zq = __uint_as_float(key << (31 - DB));
     if (!(zq > 0.0f)) return __int_as_float(0x7f800000);
     return __fmul_rn(__frcp_rn(zq), 1.0f + 0x1p-10f);
 }
