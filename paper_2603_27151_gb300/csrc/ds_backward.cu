@@ -459,7 +459,7 @@ __global__ void __launch_bounds__(kTilePix, SG == 4 ? DS_MINB_BWD4 : DS_MINB_BWD
 // gradients and score weights, then the score walk over the same staged list
 // (still in shared memory when it fits one chunk) and the winner terms.  The
 // winners' depths come from the forward walk instead of being recomputed.
-template <int SG, int TW>
+template <int TW>
 __global__ void __launch_bounds__(kTilePix, DS_MINB_TRAIN)
     k_raster_train(const __grid_constant__ ViewTable vt, const SoupDev s, const SetupRec* __restrict__ recs,
                    const uint32_t* __restrict__ keys, const uint32_t* __restrict__ vals,
@@ -488,52 +488,34 @@ __global__ void __launch_bounds__(kTilePix, DS_MINB_TRAIN)
         const ViewDesc& V = vt.v[wi.v];
         const int px = wi.tx * TW + lx, py = wi.ty * TH + ly;
         const bool valid = px < V.W && py < V.H;
-        const int s0 = wi.g * kSampleGroup;
-        const int ns = min(SG, vt.S - s0);
         const uint2 seed = view_seed(vt, wi.v);
         const size_t HW = (size_t)V.H * V.W, pix = (size_t)py * V.W + px;
 
-        int bt[SG];
-        float brho[SG], bb1[SG], bb2[SG], bD[SG];
-#pragma unroll
-        for (int q = 0; q < SG; ++q) {
-            bt[q] = -1;
-            brho[q] = 0.0f;
-            bb1[q] = bb2[q] = 0.0f;
-            bD[q] = __int_as_float(0x7f800000);
-        }
+        // the walks take arrays over a group's samples
+        int bt[1] = {-1};
+        float brho[1] = {0.0f}, bb1[1] = {0.0f}, bb2[1] = {0.0f}, bD[1] = {__int_as_float(0x7f800000)};
         const uint2 rg = ranges[V.tile_base + wi.ty * V.tiles_x + wi.tx];
-        const bool fits = forward_walk<SG, TW>(sm, recs, keys, vals, rg, DB, vt.chunk, (size_t)wi.v * s.T, wi, s, tid,
-                                               lx, ly, warp, valid, px, py, ns, seed, stochastic, bt, brho, bb1, bb2,
-                                               bD);
+        const bool fits = forward_walk<1, TW>(sm, recs, keys, vals, rg, DB, vt.chunk, (size_t)wi.v * s.T, wi, s, tid,
+                                              lx, ly, warp, valid, px, py, 1, seed, stochastic, bt, brho, bb1, bb2, bD);
 
-        // ---- G-buffer, colours, loss, upstream gradients, score weights
-        float wsc[SG];
-        bool any_score = false;
-        const int Co = s.C - 1;
-#pragma unroll
-        for (int q = 0; q < SG; ++q) {
-            wsc[q] = 0.f;
-            if (!valid || q >= ns) continue;
-            const int sg = s0 + q;
-            reinterpret_cast<int4*>(V.gbuf)[sg * HW + pix] =
-                make_int4(bt[q], __float_as_int(bb1[q]), __float_as_int(bb2[q]), __float_as_int(bD[q]));
-            const float ell = color_loss_out<false>(s, bt[q], bb1[q], bb2[q], bg, V.target + pix,
-                                             V.color + (size_t)sg * Co * HW + pix,
-                                             const_cast<float*>(V.grad_color) + (size_t)sg * Co * HW + pix, HW,
-                                             two_scale);
+        // ---- G-buffer, colour, loss, upstream gradient, score weight
+        float wsc[1] = {0.f};
+        if (valid) {
+            reinterpret_cast<int4*>(V.gbuf)[pix] =
+                make_int4(bt[0], __float_as_int(bb1[0]), __float_as_int(bb2[0]), __float_as_int(bD[0]));
+            const float ell = color_loss_out<false>(s, bt[0], bb1[0], bb2[0], bg, V.target + pix, V.color + pix,
+                                                    const_cast<float*>(V.grad_color) + pix, HW, two_scale);
             const float w = __fmul_rn(scale, ell);
-            if (V.score_w) const_cast<float*>(V.score_w)[sg * HW + pix] = w;
+            if (V.score_w) const_cast<float*>(V.score_w)[pix] = w;
             lsum += ell;
-            if (do_score) wsc[q] = w;
-            any_score = any_score || wsc[q] != 0.f;
+            if (do_score) wsc[0] = w;
         }
 
         // ---- Algorithm A1 step 2 (texture, score, interior)
-        score_walk<SG, TW>(sm, recs, keys, vals, rg, DB, vt.chunk, (size_t)wi.v * s.T, wi, s, acc_tex, tid, lx, ly,
-                           warp, fits, any_score, bt, brho, wsc, s_jobs[warp].ring);
-        winner_terms<SG, TW>(s, acc_tex, acc_verts, geom + (size_t)wi.v * s.T, view_cam(vt, wi.v), V, wi, s0, ns, HW,
-                             valid, do_tex, do_score, do_int, bt, wsc, s_jobs[warp].winners);
+        score_walk<1, TW>(sm, recs, keys, vals, rg, DB, vt.chunk, (size_t)wi.v * s.T, wi, s, acc_tex, tid, lx, ly,
+                          warp, fits, wsc[0] != 0.f, bt, brho, wsc, s_jobs[warp].ring);
+        winner_terms<1, TW>(s, acc_tex, acc_verts, geom + (size_t)wi.v * s.T, view_cam(vt, wi.v), V, wi, 0, 1, HW,
+                            valid, do_tex, do_score, do_int, bt, wsc, s_jobs[warp].winners);
         __syncthreads();
     }
     // ---- the loss: one atomic per CTA
@@ -905,9 +887,9 @@ cudaError_t launch_raster_train(const ViewTable& vt, const SoupDev& s, const Set
         kernel<<<resident_grid(kernel, vt.n_items, grid), kTilePix, 0, st>>>(
             vt, s, recs, keys, vals, ranges, DB, mode, bg, scale, loss, flags, geom, acc_tex, acc_verts, counter);
     };
-    if (vt.tile_w == 8) run(k_raster_train<1, 8>);
-    else if (vt.tile_w == 32) run(k_raster_train<1, 32>);
-    else run(k_raster_train<1, 16>);
+    if (vt.tile_w == 8) run(k_raster_train<8>);
+    else if (vt.tile_w == 32) run(k_raster_train<32>);
+    else run(k_raster_train<16>);
     note_launches(1);
     return cudaGetLastError();
 }
