@@ -631,13 +631,16 @@ __global__ void __launch_bounds__(256) k_loss_l1_ssim_tile(const __grid_constant
     }
 }
 
-// CTAs of the call with segments of `steps` steps.
-long long ssim_ctas(int n_views, int S, const int* hw, int steps) {
-    const int rows = kStep * steps - 4 * kR;
-    long long n = 0;
-    for (int v = 0; v < n_views; ++v)
-        n += (long long)S * ((hw[2 * v] + kTX - 1) / kTX) * ((hw[2 * v + 1] + rows - 1) / rows);
-    return n;
+constexpr int segment_rows(int steps) { return kStep * steps - 4 * kR; }
+
+// Adds the march's CTAs for a view with segments of K, K + 1, ... steps (K a
+// constant, so that no division is left: the host has 64 views times 8 to do
+// before the launch).
+template <int K = 2>
+void add_march_ctas(int w, int h, long long* ctas) {
+    constexpr int rows = segment_rows(K);
+    ctas[K] += (long long)((w + kTX - 1) / kTX) * ((h + rows - 1) / rows);
+    if constexpr (K < kMaxSteps) add_march_ctas<K + 1>(w, h, ctas);
 }
 
 }  // namespace
@@ -664,10 +667,12 @@ cudaError_t launch_loss_l1_ssim(int n_views, int S, int Co, const int* hw, const
     // in proportion to its steps, so the waves of CTAs times the steps (and a
     // bit for starting up) is what is least.
     const int sms = persistent_grid(1 << 30, 1);
+    long long ctas[kMaxSteps + 1] = {};
+    for (int v = 0; v < n_views; ++v) add_march_ctas(hw[2 * v], hw[2 * v + 1], ctas);
     int steps = 2;
     double best = 1e300;
     for (int k = 2; k <= kMaxSteps; ++k) {
-        const double cost = (double)((ssim_ctas(n_views, S, hw, k) + sms - 1) / sms) * (k + 0.5);
+        const double cost = (double)((S * ctas[k] + sms - 1) / sms) * (k + 0.5);
         if (cost < best) best = cost, steps = k;
     }
     const auto tiles = [](int w, int h) {
@@ -684,7 +689,7 @@ cudaError_t launch_loss_l1_ssim(int n_views, int S, int Co, const int* hw, const
     // 512 x 16).
     const long long left = n_tiles % (2 * sms);
     const bool small = 2.3 * (double)(n_tiles / (2 * sms)) + (left == 0 ? 0.0 : left <= sms ? 1.6 : 2.6) <= best;
-    t->rows = kStep * steps - 4 * kR;
+    t->rows = segment_rows(steps);
     long long cta = 0;
     for (int v = 0; v < n_views; ++v) {
         SsimView& d = t->v[v];
