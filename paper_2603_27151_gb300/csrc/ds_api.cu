@@ -145,19 +145,23 @@ namespace {
 
 constexpr int kCounters = 5;
 
-// Pairs that every list buffer holds.
+// Pairs that every buffer of the lists holds (0 after a failed allocation of
+// one of them).
 uint32_t pair_capacity(const ds_ctx* c) {
-    size_t n = std::min(std::min(c->keys[0].cap, c->keys[1].cap), std::min(c->vals[0].cap, c->vals[1].cap)) / 4;
-    return (uint32_t)std::min<size_t>(n, 0xffffffffu);
+    const size_t n = std::min(std::min(c->keys[0].cap, c->keys[1].cap), std::min(c->vals[0].cap, c->vals[1].cap)) / 4;
+    const bool chunks = c->chunks.cap >= sizeof(uint2) * ds::max_chunks(n);
+    return chunks ? (uint32_t)std::min<size_t>(n, 0xffffffffu) : 0;
 }
 
 // List buffers for at least K pairs.
 ds_status ensure_pairs(ds_ctx* c, size_t K) {
+    size_t n = SIZE_MAX;
     for (int b = 0; b < 2; ++b) {
         DS_TRY(c->keys[b].ensure(4 * K, "bin keys"));
         DS_TRY(c->vals[b].ensure(4 * K, "bin values"));
+        n = std::min(n, std::min(c->keys[b].cap, c->vals[b].cap) / 4);
     }
-    return c->chunks.ensure(sizeof(uint2) * ds::max_chunks(pair_capacity(c)), "list chunks");
+    return c->chunks.ensure(sizeof(uint2) * ds::max_chunks(n), "list chunks");
 }
 
 struct DeviceGuard {
