@@ -53,13 +53,12 @@ def test_few_tiles_are_not_waited_for(ctx):
     for w, h in ((256, 256), (1920, 1080)):
         cams = [I.look_at([0.0, 0.0, 3.0], w, h)]
         g, col, _ = N.alloc_outputs(cams, 1, 4, "cuda")
-        for k in range(6):
-            if k == 1:
-                ctx.profile_reset()
-                ctx.profile(True)
+        for _ in range(6):   # the first one sizes the buffers
+            ctx.profile_reset()
+            ctx.profile(True)
             ctx.raster_forward(sid, cams, I.mask_seeds(3, 1), 1, 0, np.zeros(3, np.float32), g, col)
-        torch.cuda.synchronize()
-        ctx.profile(False)
-        st = ctx.profile_read()
-        ms[w] = (st["setup"][1] + st["emit"][1]) / 5
+            torch.cuda.synchronize()
+            ctx.profile(False)
+            st = ctx.profile_read()
+            ms[w] = min(ms.get(w, 1e30), st["setup"][1] + st["emit"][1])
     assert ms[256] < 1.2 * ms[1920], ms

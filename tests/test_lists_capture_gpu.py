@@ -1,5 +1,9 @@
 """Long lists without a host wait: captured in a graph, with buffers that are too
 small, and after a call that a capture refuses."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -10,13 +14,7 @@ from tests.gpu_helpers import assert_forward_equal, gpu_forward
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def scene():
-    torch = pytest.importorskip("torch")
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    import __graft_entry__
-    __graft_entry__.build()
+def _scene():
     rng = np.random.default_rng(2)
     T = 5000   # lists of up to about 5,000 triangles
     verts = (rng.uniform(-0.1, 0.1, (T, 1, 3)) + rng.uniform(-0.5, 0.5, (T, 3, 3))).astype(np.float32)
@@ -24,6 +22,16 @@ def scene():
     tex[..., 3] -= 2.0
     sc = I.Scene(verts, tex, 2, [I.look_at([0.0, 0.0, 2.0], 45, 40)], I.mask_seeds(3, 1), 1, np.zeros(3, np.float32))
     return sc, O.forward(sc.verts, sc.tex, sc.grid_n, sc.cams, sc.seeds, bg=sc.bg)
+
+
+@pytest.fixture(scope="module")
+def scene():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    return _scene()
 
 
 def _result(N, g, col):
@@ -76,10 +84,10 @@ def test_buffers_too_small(scene, pairs):
     ctx.close()
 
 
-def test_waiting_call_is_refused_under_capture(scene):
+def _refused_capture():
     import torch
     from paper_2603_27151_gb300 import native as N
-    sc, ref = scene
+    sc, ref = _scene()
     ctx = N.Context(0)
     sid, _, _ = gpu_forward(ctx, sc)
     g, col, _ = N.alloc_outputs(sc.cams, 1, 4, "cuda")
@@ -96,3 +104,13 @@ def test_waiting_call_is_refused_under_capture(scene):
     torch.cuda.synchronize()
     assert_forward_equal(_result(N, g, col), ref)
     ctx.close()
+
+
+def test_waiting_call_is_refused_under_capture(scene):
+    """A call that waits for the host ends the capture with an error, and the
+    context goes on.  In a process of its own: torch's random generators stay in
+    the state of the failed capture."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    code = "from tests.test_lists_capture_gpu import _refused_capture as f; f()"
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]

@@ -70,12 +70,11 @@ def test_few_long_lists_are_sorted_side_by_side(ctx):
     for px in (64, 512):
         cams = [I.look_at([0.0, 0.0, 3.0], px, px)]
         g, col, _ = N.alloc_outputs(cams, 1, 4, "cuda")
-        for k in range(4):
-            if k == 1:
-                ctx.profile_reset()
-                ctx.profile(True)
+        for _ in range(5):   # the first one sizes the buffers
+            ctx.profile_reset()
+            ctx.profile(True)
             ctx.raster_forward(sid, cams, I.mask_seeds(3, 1), 1, 0, np.zeros(3, np.float32), g, col)
-        torch.cuda.synchronize()
-        ctx.profile(False)
-        ms[px] = ctx.profile_read()["sort"][1] / 3
+            torch.cuda.synchronize()
+            ctx.profile(False)
+            ms[px] = min(ms.get(px, 1e30), ctx.profile_read()["sort"][1])
     assert ms[64] < 4 * ms[512], ms

@@ -61,13 +61,13 @@ def test_few_wide_triangles_do_not_wait_for_a_warp(ctx, T, n, limit):
     sid = ctx.soup_upload(torch.from_numpy(verts).cuda(), tex, 1)
     cams = [I.look_at([0.0, 0.0, 3.0], 1280, 720)]
     g, col, _ = N.alloc_outputs(cams, 1, 4, "cuda")
-    for k in range(4):
-        if k == 1:
-            ctx.profile_reset()
-            ctx.profile(True)
+    ms = {}
+    for _ in range(5):   # the first one sizes the buffers
+        ctx.profile_reset()
+        ctx.profile(True)
         ctx.raster_forward(sid, cams, I.mask_seeds(3, 1), 1, 0, np.zeros(3, np.float32), g, col)
-    torch.cuda.synchronize()
-    ctx.profile(False)
-    ms = {k: v[1] / 3 for k, v in ctx.profile_read().items()}
+        torch.cuda.synchronize()
+        ctx.profile(False)
+        ms = {k: min(ms.get(k, 1e30), v[1]) for k, v in ctx.profile_read().items()}
     assert ctx.plan_stats()[0] > 1000 * n
     assert ms["setup"] + ms["emit"] < limit * ms["raster_fwd"], ms
