@@ -35,8 +35,9 @@ constexpr int kCtaBoxes = 64;     // as many of them as the CTA's list holds
 // 1280 x 720: k_setup 394 -> 32 us, k_emit 511 -> 41).  Sixteen warps per SM
 // cost 1.5 us on 16,000 records.
 static int records_per_warp(long long n_records) {
+    const long long warps = persistent_grid(1 << 30, 8);
     int per = 1;
-    while (per < 32 && n_records > (long long)per * persistent_grid(1 << 30, 8)) per *= 2;
+    while (per < 32 && n_records > per * warps) per *= 2;
     return per;
 }
 
@@ -114,7 +115,9 @@ __device__ __forceinline__ void for_tiles(const ViewTable& vt, int per, int v, c
         cta = at < kCtaBoxes;
         if (cta) s_box[at] = CtaBox{r, box, v, t, zkey};
     }
-    const int own = max(4, kOwnTiles * per / 32);   // fewer records per warp: more lanes idle
+    // by itself a lane takes nb / 4 rounds, beside the others; shared, a box takes
+    // one of the warp's, after the others
+    const int own = min(kOwnTiles, 4 * per);
     if (nb <= own) walk(r, v, box.x, box.y, box.z - box.x + 1, 0, 1, nb, t, zkey);
     unsigned wide = __ballot_sync(kFull, nb > own && !cta);
     while (wide) {
@@ -608,8 +611,9 @@ cudaError_t launch_tile_sort(const ViewTable& vt, const uint2* ranges, int n_til
     // Few tiles: fewer of them per CTA, down to one, so that their lists are
     // sorted side by side (eight always: b 24 -> 50, 256 tiles of 740 entries
     // 28 -> 53).  Up to four CTAs per SM; two or eight measure alike.
+    const int ctas = persistent_grid(1 << 30, 4);
     int per = 1;
-    while (per < kSortWarps && n_tiles > per * persistent_grid(1 << 30, 4)) per *= 2;
+    while (per < kSortWarps && n_tiles > per * ctas) per *= 2;
     const bool lng = long_lists(vt);
     const int grid = std::max((n_tiles + per - 1) / per, lng ? chunk_grid(cap) : 1);
     k_tile_sort<<<grid, kSortThreads, 0, st>>>(ranges, n_tiles, per, DB, lng ? n_chunks : nullptr, chunks, k0, v0, k1, v1);
