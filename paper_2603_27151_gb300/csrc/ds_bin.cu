@@ -10,8 +10,9 @@
 // are no depth bits: the forward's results do not depend on the order (its
 // tie-break is by triangle index), but the backward sums the opacity terms of
 // neighbouring list entries in FP32 before the FP64 accumulators, and those
-// groups have to be the same in every call.  A call makes 4 launches here
-// (5 above 4,096 tiles) and a memset.  The radix sort of (tile, depth) keys that
+// groups have to be the same in every call.  A call makes 4 launches here (5
+// above 4,096 tiles, one more where a list is above 2,048 entries or, without
+// a host wait, can be) and a memset.  The radix sort of (tile, depth) keys that
 // this replaces made 4 passes of 5 launches over all pairs: 146 us of a
 // 1.28 ms training step (239,566 pairs), 39 us of a 120 us render of 64
 // triangles.

@@ -151,7 +151,7 @@ __device__ __forceinline__ void stage_coarse(float* zs, const float* __restrict_
 // small stages keep five CTAs resident per SM.  Issue-bound (77% of the slots
 // at 423 instructions per item of four channels): the interpolation, the sums
 // and the sigmoid's exponential run on packed pairs of channels, with the
-// sigmoid's range test once per item (323 instructions; levels 2..5 of 20,000
+// sigmoid's range test once per item (321 instructions; levels 2..5 of 20,000
 // triangles 326 -> 265 us; six CTAs 277, CTAs of 128 or 192 threads 265).
 template <bool kAct>
 __global__ void __launch_bounds__(256, 5) k_compose(const float* __restrict__ levels, int T, int r_min, int r_max,
