@@ -84,6 +84,20 @@ def test_buffers_too_small(scene, pairs):
     ctx.close()
 
 
+def test_without_allocation(scene):
+    """The allocation-free forward on the same lists, twice on its scratch."""
+    import torch
+    from paper_2603_27151_gb300 import native as N
+    sc, ref = scene
+    v, t = torch.from_numpy(sc.verts).cuda(), torch.from_numpy(sc.tex).cuda()
+    g, col, _ = N.alloc_outputs(sc.cams, 1, 4, "cuda")
+    for _ in range(2):
+        g[0].fill_(-7)
+        N.raster_forward_noalloc(v, t, sc.grid_n, sc.cams, sc.seeds, 1, 0, sc.bg, g, col)
+        torch.cuda.synchronize()
+        assert_forward_equal(_result(N, g, col), ref)
+
+
 def _refused_capture():
     import torch
     from paper_2603_27151_gb300 import native as N
