@@ -3,19 +3,18 @@
 //
 // The set-up kernel counts the triangles of every tile (k_setup); the counts
 // are scanned over the tiles; k_emit places each (tile, triangle) pair at its
-// tile's cursor, in whatever order its atomics are served; k_tile_sort then
-// (with k_list_merge for lists above 2,048 entries) gives every list its one
-// order.  The early exit of the walks wants it front
-// to back.  The triangle index breaks ties, and is the whole key when there
-// are no depth bits: the forward's results do not depend on the order (its
-// tie-break is by triangle index), but the backward sums the opacity terms of
-// neighbouring list entries in FP32 before the FP64 accumulators, and those
-// groups have to be the same in every call.  A call makes 4 launches here (5
-// above 4,096 tiles, one more where a list is above 2,048 entries or, without
-// a host wait, can be) and a memset.  The radix sort of (tile, depth) keys that
-// this replaces made 4 passes of 5 launches over all pairs: 146 us of a
-// 1.28 ms training step (239,566 pairs), 39 us of a 120 us render of 64
-// triangles.
+// tile's cursor, in whatever order its atomics are served; k_tile_sort (with
+// k_list_merge for lists above 2,048 entries) then gives every list its one
+// order.  The early exit of the walks wants it front to back.  The triangle
+// index breaks ties, and is the whole key when there are no depth bits: the
+// forward's results do not depend on the order (its tie-break is by triangle
+// index), but the backward sums the opacity terms of neighbouring list entries
+// in FP32 before the FP64 accumulators, and those groups have to be the same in
+// every call.  A call makes 4 launches here (5 above 4,096 tiles, one more
+// where a list is above 2,048 entries or, without a host wait, can be) and a
+// memset.  The radix sort of (tile, depth) keys that this replaces made 4
+// passes of 5 launches over all pairs: 146 us of a 1.28 ms training step
+// (239,566 pairs), 39 us of a 120 us render of 64 triangles.
 #include <algorithm>
 
 #include "ds_internal.h"
@@ -25,7 +24,7 @@ namespace ds {
 namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kBinThreads = 256;
-constexpr int kOwnTiles = 32;     // boxes of more tiles are shared by the warp,
+constexpr int kOwnTiles = 32;     // boxes of more tiles are shared by the warp (16 and 64 measure alike),
 constexpr int kWarpTiles = 1024;  // those of more than this by the CTA
 constexpr int kCtaBoxes = 64;     // as many of them as the CTA's list holds
 }  // namespace
@@ -155,10 +154,10 @@ __device__ __forceinline__ int view_of_record(const ViewTable& vt, long long gid
     return v;
 }
 
-// One thread per (view, triangle), `per` of them in a warp: project, snap to 1/256 pixel, cull, build
-// the oriented edge functions with the top-left fill rule (Eq. 1 fragments),
-// the perspective factors k_i and the tile rectangle, and count the triangle
-// in every tile whose pixel centres it may cover.
+// One thread per (view, triangle), `per` of them in a warp: project, snap to
+// 1/256 pixel, cull, build the oriented edge functions with the top-left fill
+// rule (Eq. 1 fragments), the perspective factors k_i and the tile rectangle,
+// and count the triangle in every tile whose pixel centres it may cover.
 __global__ void __launch_bounds__(kBinThreads) k_setup(const __grid_constant__ ViewTable vt, long long n_records, int per,
                                                        bool split, SetupRec* __restrict__ recs, uint32_t* __restrict__ tile_count,
                                                        int4* __restrict__ tbox, uint32_t* __restrict__ zkeys) {

@@ -23,7 +23,9 @@ constexpr int kBlkW = 8, kBlkH = 4;              // a warp's pixels
 constexpr int kBlocksPerTile = kTilePix / 32;    // 8 in every tile shape
 constexpr int kStage = 32;                       // staged triangles per warp and round
 constexpr int kWarps = kTilePix / 32;            // warps of a CTA
-constexpr int kExitEvery = 4;                    // staged triangles between two votes on the early exit
+// Staged triangles between two votes on the early exit (200,000 triangles at
+// 1080p, binary opacity: every one 160 us, 2: 154, 4: 150, 8 and 16: 148).
+constexpr int kExitEvery = 4;
 
 // A warp's staged set-up: TileStage's terms relative to the block's first
 // pixel.
