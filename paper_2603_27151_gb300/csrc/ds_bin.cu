@@ -433,27 +433,27 @@ cudaError_t launch_emit(const ViewTable& vt, int n_tiles, const SetupRec* recs, 
 namespace {
 constexpr int kSortWarps = 8;       // most tiles per CTA of k_tile_sort
 constexpr int kWarpList = 128;      // lists up to this length: one warp, in registers (64: a 76 -> 109, b 24 -> 11)
+constexpr int kWarpTriangles = 256; // the same without depth keys
 constexpr int kSortThreads = 256;   // 512: a 76 -> 99, d 51 -> 45
 }  // namespace
 
 // Ranks of E entries per lane among the warp's n by counting the smaller ones
-// ((key, triangle) pairs are distinct), written back in order; kKeys: there
-// are depth keys.
-template <int E, bool kKeys>
+// ((key, triangle) pairs are distinct), written back in order.
+template <int E>
 __device__ __forceinline__ void sort_warp(uint32_t* keys, uint32_t* vals, uint32_t lo, int n, int lane) {
     uint32_t k[E], v[E];
     int rank[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         const bool in = lane + 32 * e < n;
-        k[e] = kKeys && in ? keys[lo + lane + 32 * e] : 0u;
+        k[e] = in ? keys[lo + lane + 32 * e] : 0u;
         v[e] = in ? vals[lo + lane + 32 * e] : 0u;
         rank[e] = 0;
     }
 #pragma unroll
     for (int f = 0; f < E; ++f)
         for (int j = 0; j < min(32, n - 32 * f); ++j) {
-            const uint32_t kj = kKeys ? __shfl_sync(kFull, k[f], j) : 0u, vj = __shfl_sync(kFull, v[f], j);
+            const uint32_t kj = __shfl_sync(kFull, k[f], j), vj = __shfl_sync(kFull, v[f], j);
 #pragma unroll
             for (int e = 0; e < E; ++e) rank[e] += kj < k[e] || (kj == k[e] && vj < v[e]) ? 1 : 0;
         }
@@ -461,16 +461,53 @@ __device__ __forceinline__ void sort_warp(uint32_t* keys, uint32_t* vals, uint32
 #pragma unroll
     for (int e = 0; e < E; ++e)
         if (lane + 32 * e < n) {
-            if (kKeys) keys[lo + rank[e]] = k[e];
+            keys[lo + rank[e]] = k[e];
             vals[lo + rank[e]] = v[e];
         }
 }
 
+// Without depth keys: a bitonic network over the triangles in the warp's 32 E
+// registers (the 1080p batch's 1.6 M pairs: counting as above 49 us, the network
+// 39, and up to 256 entries in a warp 30).
+template <int E>
+__device__ __forceinline__ void sort_warp_triangles(uint32_t* vals, uint32_t lo, int n, int lane) {
+    uint32_t v[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = lane + 32 * e < n ? vals[lo + lane + 32 * e] : 0xffffffffu;
+#pragma unroll
+    for (int k = 2; k <= 32 * E; k <<= 1)
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1)
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const bool up = ((lane + 32 * e) & k) == 0;
+                if (j < 32) {   // the partner is the same register of another lane
+                    const uint32_t o = __shfl_xor_sync(kFull, v[e], j);
+                    v[e] = ((lane & j) == 0) == up ? min(v[e], o) : max(v[e], o);
+                } else if (!(e & (j >> 5))) {   // another register of this lane
+                    const int p = e | (j >> 5);
+                    const uint32_t a = min(v[e], v[p]), b = max(v[e], v[p]);
+                    v[e] = up ? a : b;
+                    v[p] = up ? b : a;
+                }
+            }
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if (lane + 32 * e < n) vals[lo + lane + 32 * e] = v[e];
+}
+
 template <bool kKeys>
 __device__ __forceinline__ void sort_short(uint32_t* keys, uint32_t* vals, uint32_t lo, int n, int lane) {
-    if (n > 64) sort_warp<4, kKeys>(keys, vals, lo, n, lane);
-    else if (n > 32) sort_warp<2, kKeys>(keys, vals, lo, n, lane);
-    else if (n > 1) sort_warp<1, kKeys>(keys, vals, lo, n, lane);
+    if constexpr (kKeys) {
+        if (n > 64) sort_warp<4>(keys, vals, lo, n, lane);
+        else if (n > 32) sort_warp<2>(keys, vals, lo, n, lane);
+        else if (n > 1) sort_warp<1>(keys, vals, lo, n, lane);
+    } else {
+        if (n > 128) sort_warp_triangles<8>(vals, lo, n, lane);
+        else if (n > 64) sort_warp_triangles<4>(vals, lo, n, lane);
+        else if (n > 32) sort_warp_triangles<2>(vals, lo, n, lane);
+        else if (n > 1) sort_warp_triangles<1>(vals, lo, n, lane);
+    }
 }
 
 // n <= kBlockList entries (depth key, triangle) from k, v in order into ko, vo
@@ -503,15 +540,16 @@ __device__ __forceinline__ void sort_block(unsigned long long* s_kv, const uint3
 }
 
 // Every tile's list by (depth key, triangle).  Most lists are short (a few
-// dozen triangles): one warp each.  The CTA then takes its tiles with lists
-// above kWarpList one after the other, and of the lists above kBlockList its
+// dozen triangles): one warp each.  The CTA then takes its tiles with longer
+// lists one after the other, and of the lists above kBlockList its
 // share of the chunks, which go to (k1, v1) for k_list_merge.  A CTA's `per`
 // tiles are gridDim.x apart, since long lists come in neighbouring tiles.
 // Bound by the latency of the network's stages (c) or by shared memory (e).
 // With eight tiles to every CTA and lists above 2,048 entries in radix passes
 // of one CTA: b 49, c 137, d 582, e 2,029 us; now 24, 51, 51 and 132 (a global
 // radix sort of all pairs: 64, 80, 109 and 117, and a 171 against 76).
-__global__ void __launch_bounds__(kSortThreads) k_tile_sort(const uint2* __restrict__ ranges, int n_tiles, int per, int DB,
+template <bool kKeys>   // there are depth keys
+__global__ void __launch_bounds__(kSortThreads) k_tile_sort(const uint2* __restrict__ ranges, int n_tiles, int per,
                                                             const uint32_t* __restrict__ n_chunks,
                                                             const uint2* __restrict__ chunks, uint32_t* __restrict__ k0,
                                                             uint32_t* __restrict__ v0, uint32_t* __restrict__ k1,
@@ -519,26 +557,26 @@ __global__ void __launch_bounds__(kSortThreads) k_tile_sort(const uint2* __restr
     __shared__ unsigned long long s_kv[kBlockList];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     bool lng = false;
+    constexpr int kShort = kKeys ? kWarpList : kWarpTriangles;
     const int tile = blockIdx.x + warp * gridDim.x;
     if (warp < per && tile < n_tiles) {
         const uint2 rg = ranges[tile];
         const int n = (int)(rg.y - rg.x);
-        if (n > kWarpList) lng = true;
-        else if (DB > 0) sort_short<true>(k0, v0, rg.x, n, lane);
-        else sort_short<false>(k0, v0, rg.x, n, lane);
+        if (n > kShort) lng = true;
+        else sort_short<kKeys>(k0, v0, rg.x, n, lane);
     }
     const bool any = __syncthreads_or(lng);
     for (int q = 0; any && q < per; ++q) {
         if ((int)(blockIdx.x + q * gridDim.x) >= n_tiles) break;
         const uint2 rg = ranges[blockIdx.x + q * gridDim.x];
         const int n = (int)(rg.y - rg.x);
-        if (n > kWarpList && n <= kBlockList) sort_block(s_kv, k0 + rg.x, v0 + rg.x, k0 + rg.x, v0 + rg.x, n, DB > 0);
+        if (n > kShort && n <= kBlockList) sort_block(s_kv, k0 + rg.x, v0 + rg.x, k0 + rg.x, v0 + rg.x, n, kKeys);
     }
     const uint32_t nc = n_chunks ? *n_chunks : 0u;
     for (uint32_t i = blockIdx.x; i < nc; i += gridDim.x) {
         const uint2 ch = chunks[i], rg = ranges[ch.x];
         const uint32_t lo = rg.x + ch.y * kBlockList;
-        sort_block(s_kv, k0 + lo, v0 + lo, k1 + lo, v1 + lo, (int)min((uint32_t)kBlockList, rg.y - lo), DB > 0);
+        sort_block(s_kv, k0 + lo, v0 + lo, k1 + lo, v1 + lo, (int)min((uint32_t)kBlockList, rg.y - lo), kKeys);
     }
 }
 
@@ -616,7 +654,8 @@ cudaError_t launch_tile_sort(const ViewTable& vt, const uint2* ranges, int n_til
     while (per < kSortWarps && n_tiles > per * ctas) per *= 2;
     const bool lng = long_lists(vt);
     const int grid = std::max((n_tiles + per - 1) / per, lng ? chunk_grid(cap) : 1);
-    k_tile_sort<<<grid, kSortThreads, 0, st>>>(ranges, n_tiles, per, DB, lng ? n_chunks : nullptr, chunks, k0, v0, k1, v1);
+    const auto kernel = DB > 0 ? k_tile_sort<true> : k_tile_sort<false>;
+    kernel<<<grid, kSortThreads, 0, st>>>(ranges, n_tiles, per, lng ? n_chunks : nullptr, chunks, k0, v0, k1, v1);
     note_launches(1);
     return cudaGetLastError();
 }
